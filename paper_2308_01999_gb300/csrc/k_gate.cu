@@ -30,6 +30,7 @@
 #include <type_traits>
 #include <vector>
 
+#include "k_common.cuh"
 #include "sv_internal.h"
 
 namespace svk {
@@ -38,44 +39,9 @@ namespace {
 enum Mode { PAIR = 0, T0 = 1, SCALAR = 2 };
 constexpr int kThreads = 256;
 
-template <typename R> struct CT;
-template <> struct CT<float> { using T = float2; };
-template <> struct CT<double> { using T = double2; };
-
-__device__ __forceinline__ float fmac(float a, float b, float c) { return __fmaf_rn(a, b, c); }
-__device__ __forceinline__ double fmac(double a, double b, double c) { return __fma_rn(a, b, c); }
-
-// acc += m * v (complex)
-template <typename C>
-__device__ __forceinline__ void cmad(C &acc, const C &m, const C &v) {
-    acc.x = fmac(m.x, v.x, acc.x);
-    acc.x = fmac(-m.y, v.y, acc.x);
-    acc.y = fmac(m.x, v.y, acc.y);
-    acc.y = fmac(m.y, v.x, acc.y);
-}
-
-template <typename C>
-__device__ __forceinline__ C cmul(const C &a, const C &b) {
-    C r;
-    r.x = fmac(a.x, b.x, -a.y * b.y);
-    r.y = fmac(a.x, b.y, a.y * b.x);
-    return r;
-}
-
-// Zero bits inserted at G.pos (ascending), then the control bits set.
-__device__ __forceinline__ uint64_t insert_zeros(uint64_t g, const GroupGeom &G) {
-#pragma unroll 1
-    for (int i = 0; i < G.ns; ++i) {
-        const uint64_t lo = g & ((1ull << G.pos[i]) - 1ull);
-        g = ((g ^ lo) << 1) | lo;
-    }
-    return g | G.cset;
-}
-
 __device__ __forceinline__ float4 ld16(const float2 *p) { return *reinterpret_cast<const float4 *>(p); }
 __device__ __forceinline__ void st16(float2 *p, const float4 &v) { *reinterpret_cast<float4 *>(p) = v; }
 
-template <int K> struct Offs { uint64_t o[1 << K]; };
 template <typename R, int K> struct MatK { typename CT<R>::T m[1 << (2 * K)]; };
 
 // ---------------------------------------------------------------------------
@@ -803,6 +769,10 @@ cudaError_t dense6_c64(const LaunchCtx &L, void *sv, int n, const GroupGeom &G, 
 template <typename R>
 cudaError_t dense_any(const LaunchCtx &L, void *sv, int n, const GroupGeom &G, const int *tpos, int k,
                       const double *mat, void *d_mat) {
+    if constexpr (std::is_same<R, double>::value) {
+        cudaError_t e;
+        if (try_dense_fx(L, sv, n, G, tpos, k, mat, e)) return e;
+    }
     switch (k) {
     case 1: return dense_reg<R, 1>(L, sv, n, G, tpos, mat);
     case 2: return dense_reg<R, 2>(L, sv, n, G, tpos, mat);
