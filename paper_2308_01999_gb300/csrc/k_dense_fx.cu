@@ -26,7 +26,7 @@
 // the exponent) is computed in FP64 in the same kernel, with k_dense's sums in
 // k_dense's order.
 #include <cmath>
-#include <cstring>
+#include <vector>
 
 #include "k_common.cuh"
 #include "sv_internal.h"
@@ -57,6 +57,14 @@ __device__ __forceinline__ double pack(uint64_t v, int be, int s) {
     m += (lo >> 10) & 1u;
     const uint32_t h = (uint32_t)(m >> 32) + ((uint32_t)(be - 1) << 20);   // the implicit bit adds one
     return __hiloint2double((int)(h | ((uint32_t)s & 0x80000000u)), (int)(uint32_t)m);
+}
+
+// An integer r times 2^sc; the caller's sc keeps the exponent in range. (The hardware conversion
+// takes one instruction where normalising by hand takes about twenty: 26-qubit
+// one-qubit gate 0.425 -> 0.326 ms.)
+__device__ __forceinline__ double scaled(double r, int sc) {
+    const int hi = __double2hiint(r);
+    return __hiloint2double(hi == 0 ? 0 : hi + (int)((uint32_t)sc << 20), __double2loint(r));
 }
 
 // mantissa of x with the implicit bit at bit 63
@@ -134,13 +142,9 @@ k_dense_fx2(double2 *__restrict__ sv, uint64_t n_groups, GroupGeom G, Offs<K> O,
             x1[i] = (int)__funnelshift_r((uint32_t)F, (uint32_t)(F >> 32), 30) * sg;
             x0[i] = (int)((uint32_t)F & 0x3fffffffu) * sg;
         }
-        const int be = E + M.em + 64 + 60 - P - PM;
+        const int sc = E - 1022 + M.em + 60 - P - PM;
         auto out = [&](long long a1, long long a0) {
-            const long long r = a1 + ((a0 + (1ll << 29)) >> 30);
-            const int s = (int)(r >> 63);
-            const uint64_t a = ((uint64_t)r ^ (uint64_t)(long long)s) - (uint64_t)(long long)s;
-            const int n = __clzll((long long)a);
-            return a == 0 ? 0.0 : pack(a << n, be - n, s);
+            return scaled(__ll2double_rn(a1 + ((a0 + (1ll << 29)) >> 30)), sc);
         };
 #pragma unroll
         for (int j = 0; j < D; ++j) {
@@ -180,6 +184,7 @@ k_dense_fx2(double2 *__restrict__ sv, uint64_t n_groups, GroupGeom G, Offs<K> O,
 // broadcast from shared memory, 24 bytes per complex product).
 // ---------------------------------------------------------------------------
 constexpr int kL = 28;
+constexpr int kFx3Threads = 128;
 
 template <int K> struct Fx3 {
     int m[1 << (2 * K)][6];          // r2, r1, r0, i2, i1, i0
@@ -191,15 +196,6 @@ template <int K> struct Fx3 {
 struct Sum3 {
     long long a2, a1, a0;
 };
-
-__device__ __forceinline__ void mul3(Sum3 &s, int x2, int x1, int x0, int m2, int m1, int m0) {
-    s.a2 = mad_wide(x2, m2, s.a2);
-    s.a1 = mad_wide(x2, m1, s.a1);
-    s.a1 = mad_wide(x1, m2, s.a1);
-    s.a0 = mad_wide(x2, m0, s.a0);
-    s.a0 = mad_wide(x1, m1, s.a0);
-    s.a0 = mad_wide(x0, m2, s.a0);
-}
 
 // a2 2^2L + a1 2^L + a0 as a double; be: biased exponent of 2^63 in units of a2
 __device__ __forceinline__ double out3(long long a2, long long a1, long long a0, int be) {
@@ -224,28 +220,37 @@ __device__ __forceinline__ double out3(long long a2, long long a1, long long a0,
     return pack(v, be - n, s);
 }
 
-template <int K>
-__global__ void __launch_bounds__(kThreads)
+// A group is shared by S lanes, DL = 2^K / S of its amplitudes each (lane s holds
+// members s DL .. s DL + DL - 1): each lane sums its members' share of S rows,
+// then hands every other lane its row's partial sums and finishes one row.
+template <int K, int S>
+__global__ void __launch_bounds__(kFx3Threads, 4)
 k_dense_fx3(double2 *__restrict__ sv, uint64_t n_groups, GroupGeom G, const __grid_constant__ Offs<K> O,
             const __grid_constant__ Fx3<K> M) {
-    constexpr int D = 1 << K;
-    __shared__ __align__(16) int Ms[D * D][8];
-    for (int i = threadIdx.x; i < D * D * 6; i += kThreads) Ms[i / 6][i % 6] = M.m[i / 6][i % 6];
+    constexpr int D = 1 << K, DL = D / S;
+    constexpr int RS = (DL * 8 + (S > 1 ? 8 : 0)) * S;   // ints of a row; lanes' parts 8 banks apart
+    __shared__ __align__(16) int Ms[D * RS];
+    for (int i = threadIdx.x; i < D * D * 6; i += kFx3Threads) {
+        const int e = i / 6, j = e / D, l = e % D;
+        Ms[j * RS + (l / DL) * (RS / S) + (l % DL) * 8 + i % 6] = M.m[e][i % 6];
+    }
     __syncthreads();
-    const uint64_t g = (uint64_t)blockIdx.x * kThreads + threadIdx.x;
-    if (g >= n_groups) return;
+    const int s = threadIdx.x & (S - 1);
+    uint64_t g = ((uint64_t)blockIdx.x * kFx3Threads + threadIdx.x) / S;
+    const bool valid = g < n_groups;
+    if (!valid) g = 0;                                  // whole warps take part in the exchanges; nothing is stored
     const uint64_t base = insert_zeros(g, G);
-    int x[2 * D][3];
+    int x[2 * DL][3];
     int E;
-    bool slow;
+    bool slow, zero;
     {
-        double2 v[D];
+        double2 v[DL];
 #pragma unroll
-        for (int j = 0; j < D; ++j) v[j] = sv[base + O.o[j]];
+        for (int j = 0; j < DL; ++j) v[j] = sv[base + O.o[s * DL + j]];
         int top = 0;
-        uint32_t low = 0xffffffffu, denorm = 0, any = 0;
+        uint32_t low = 0xffffffffu, denorm = 0;
 #pragma unroll
-        for (int l = 0; l < D; ++l) {
+        for (int l = 0; l < DL; ++l) {
             const int hr = __double2hiint(v[l].x) & 0x7fffffff, hj = __double2hiint(v[l].y) & 0x7fffffff;
             const uint32_t lw = (uint32_t)__double2loint(v[l].x) | (uint32_t)__double2loint(v[l].y);
             const int a = max(hr, hj);
@@ -253,63 +258,332 @@ k_dense_fx3(double2 *__restrict__ sv, uint64_t n_groups, GroupGeom G, const __gr
             low = min(low, (uint32_t)a - 1u);          // an exact zero wraps around and does not count
             if (a == 0) denorm |= lw;
         }
-        any = (uint32_t)top | denorm;
-        E = top >> 20;
-        slow = (unsigned)(E - kEMin) > (unsigned)(kEMax - kEMin) || denorm != 0 ||
-               (uint32_t)top - low > ((uint32_t)M.t << 20);
-        if (any == 0) return;                           // the product of zeros: the amplitudes stay zero
-        if (!slow) {
 #pragma unroll
-            for (int i = 0; i < 2 * D; ++i) {
-                const double w = (i & 1) ? v[i >> 1].y : v[i >> 1].x;
-                const int hi = __double2hiint(w);
-                const uint32_t d = (uint32_t)(E - ((hi >> 20) & 0x7ff));
-                const uint64_t m = mant64(hi, __double2loint(w));
-                const uint64_t hl = shr64(m, d);
-                const uint32_t r2 = (uint32_t)(hl >> 32), r1 = (uint32_t)hl;
-                const uint32_t r0 = d <= 32 ? shl32((uint32_t)m, 32 - d) : (uint32_t)shr64(m, d - 32);
-                constexpr uint32_t mask = (1u << kL) - 1u;
-                const int sg = (hi >> 31) | 1;
-                x[i][0] = (int)(r2 >> (32 - kL)) * sg;
-                x[i][1] = (int)(__funnelshift_r(r1, r2, 64 - 2 * kL) & mask) * sg;
-                x[i][2] = (int)(__funnelshift_r(r0, r1, 96 - 3 * kL) & mask) * sg;
+        for (int o = 1; o < S; o <<= 1) {
+            top = max(top, __shfl_xor_sync(0xffffffffu, top, o));
+            low = min(low, __shfl_xor_sync(0xffffffffu, low, o));
+            denorm |= __shfl_xor_sync(0xffffffffu, denorm, o);
+        }
+        E = top >> 20;
+        zero = ((uint32_t)top | denorm) == 0;           // the product of zeros: the amplitudes stay zero
+        slow = !zero && ((unsigned)(E - kEMin) > (unsigned)(kEMax - kEMin) || denorm != 0 ||
+                         (uint32_t)top - low > ((uint32_t)M.t << 20));
+#pragma unroll
+        for (int i = 0; i < 2 * DL; ++i) {
+            const double w = (i & 1) ? v[i >> 1].y : v[i >> 1].x;
+            const int hi = __double2hiint(w);
+            const uint32_t d = (uint32_t)(E - ((hi >> 20) & 0x7ff));
+            const uint64_t m = mant64(hi, __double2loint(w));
+            const uint64_t hl = shr64(m, d);
+            const uint32_t r2 = (uint32_t)(hl >> 32), r1 = (uint32_t)hl;
+            const uint32_t r0 = d <= 32 ? shl32((uint32_t)m, 32 - d) : (uint32_t)shr64(m, d - 32);
+            constexpr uint32_t mask = (1u << kL) - 1u;
+            const int sg = (hi >> 31) | 1;
+            x[i][0] = (int)(r2 >> (32 - kL)) * sg;
+            x[i][1] = (int)(__funnelshift_r(r1, r2, 64 - 2 * kL) & mask) * sg;
+            x[i][2] = (int)(__funnelshift_r(r0, r1, 96 - 3 * kL) & mask) * sg;
+        }
+    }
+    if (__any_sync(0xffffffffu, slow)) {
+        // lane s computes rows s DL .. s DL + DL - 1 of its group in FP64
+        double2 acc[DL];
+#pragma unroll
+        for (int j = 0; j < DL; ++j) acc[j] = make_double2(0.0, 0.0);
+        if (slow) {
+#pragma unroll 1
+            for (int l = 0; l < D; ++l) {
+                const double2 w = sv[base + O.o[l]];
+#pragma unroll
+                for (int j = 0; j < DL; ++j) cmad(acc[j], M.f[(s * DL + j) * D + l], w);
             }
         }
-    }
-    if (slow) {
-        double2 acc[D];
+        __syncwarp();                                   // every lane has read its group before any writes it
+        if (slow && valid) {
 #pragma unroll
-        for (int j = 0; j < D; ++j) acc[j] = make_double2(0.0, 0.0);
-#pragma unroll 1
-        for (int l = 0; l < D; ++l) {
-            const double2 w = sv[base + O.o[l]];
-#pragma unroll
-            for (int j = 0; j < D; ++j) cmad(acc[j], M.f[j * D + l], w);
+            for (int j = 0; j < DL; ++j) sv[base + O.o[s * DL + j]] = acc[j];
         }
-#pragma unroll
-        for (int j = 0; j < D; ++j) sv[base + O.o[j]] = acc[j];
-        return;
     }
+    if (__all_sync(0xffffffffu, slow || zero)) return;
+    const bool store = valid && !slow && !zero;
     // weight of a2: 2^(4L - 84 - 83 + E - 1022 + em); its bit 63 has biased exponent
     // that plus 63 + 1023
     const int be = E + M.em + 64 + 4 * kL - 167;
     // the row loop stays rolled (the unrolled kernel would not fit the instruction cache)
 #pragma unroll 1
-    for (int j = 0; j < D; ++j) {
-        Sum3 t1{0, 0, 0}, t2{0, 0, 0}, t3{0, 0, 0};
-        const int(*mrow)[8] = &Ms[j * D];
+    for (int j = 0; j < D; j += S) {
+        Sum3 re[S], im[S];
 #pragma unroll
-        for (int l = 0; l < D; ++l) {
-            const int4 ma = *reinterpret_cast<const int4 *>(mrow[l]);
-            const int2 mb = *reinterpret_cast<const int2 *>(mrow[l] + 4);
-            const int *a = x[2 * l], *b = x[2 * l + 1];
-            mul3(t1, a[0], a[1], a[2], ma.x, ma.y, ma.z);
-            mul3(t2, b[0], b[1], b[2], ma.w, mb.x, mb.y);
-            mul3(t3, a[0] + b[0], a[1] + b[1], a[2] + b[2], ma.x + ma.w, ma.y + mb.x, ma.z + mb.y);
+        for (int r = 0; r < S; ++r) {
+            // rounds of nine independent sums: the multiply-adds of one sum are far apart
+            Sum3 t1{0, 0, 0}, t2{0, 0, 0}, t3{0, 0, 0};
+            const int *mrow = Ms + (j + r) * RS + s * (RS / S);
+#pragma unroll
+            for (int l = 0; l < DL; ++l) {
+                const int4 ma = *reinterpret_cast<const int4 *>(mrow + 8 * l);
+                const int2 mb = *reinterpret_cast<const int2 *>(mrow + 8 * l + 4);
+                const int *a = x[2 * l], *b = x[2 * l + 1];
+                const int c2 = a[0] + b[0], c1 = a[1] + b[1], c0 = a[2] + b[2];
+                const int n2 = ma.x + ma.w, n1 = ma.y + mb.x, n0 = ma.z + mb.y;
+                t1.a2 = mad_wide(a[0], ma.x, t1.a2);
+                t2.a2 = mad_wide(b[0], ma.w, t2.a2);
+                t3.a2 = mad_wide(c2, n2, t3.a2);
+                t1.a1 = mad_wide(a[0], ma.y, t1.a1);
+                t2.a1 = mad_wide(b[0], mb.x, t2.a1);
+                t3.a1 = mad_wide(c2, n1, t3.a1);
+                t1.a0 = mad_wide(a[0], ma.z, t1.a0);
+                t2.a0 = mad_wide(b[0], mb.y, t2.a0);
+                t3.a0 = mad_wide(c2, n0, t3.a0);
+                t1.a1 = mad_wide(a[1], ma.x, t1.a1);
+                t2.a1 = mad_wide(b[1], ma.w, t2.a1);
+                t3.a1 = mad_wide(c1, n2, t3.a1);
+                t1.a0 = mad_wide(a[1], ma.y, t1.a0);
+                t2.a0 = mad_wide(b[1], mb.x, t2.a0);
+                t3.a0 = mad_wide(c1, n1, t3.a0);
+                t1.a0 = mad_wide(a[2], ma.x, t1.a0);
+                t2.a0 = mad_wide(b[2], ma.w, t2.a0);
+                t3.a0 = mad_wide(c0, n2, t3.a0);
+            }
+            re[r] = Sum3{t1.a2 - t2.a2, t1.a1 - t2.a1, t1.a0 - t2.a0};
+            im[r] = Sum3{t3.a2 - t1.a2 - t2.a2, t3.a1 - t1.a1 - t2.a1, t3.a0 - t1.a0 - t2.a0};
         }
-        const double re = out3(t1.a2 - t2.a2, t1.a1 - t2.a1, t1.a0 - t2.a0, be);
-        const double im = out3(t3.a2 - t1.a2 - t2.a2, t3.a1 - t1.a1 - t2.a1, t3.a0 - t1.a0 - t2.a0, be);
-        sv[base + O.o[j]] = make_double2(re, im);
+        // lane s keeps row j + s: at each step half of the rows go to the other lane
+#pragma unroll
+        for (int o = S / 2; o > 0; o >>= 1) {
+            const bool up = (s & o) != 0;
+#pragma unroll
+            for (int r = 0; r < o; ++r) {
+                auto trade = [&](long long &keep, long long &give) {
+                    const long long mine = up ? give : keep, send = up ? keep : give;
+                    keep = mine + __shfl_xor_sync(0xffffffffu, send, o);
+                };
+                trade(re[r].a2, re[r + o].a2);
+                trade(re[r].a1, re[r + o].a1);
+                trade(re[r].a0, re[r + o].a0);
+                trade(im[r].a2, im[r + o].a2);
+                trade(im[r].a1, im[r + o].a1);
+                trade(im[r].a0, im[r + o].a0);
+            }
+        }
+        const double2 w = make_double2(out3(re[0].a2, re[0].a1, re[0].a0, be), out3(im[0].a2, im[0].a1, im[0].a0, be));
+        if (store) sv[base + O.o[j + s]] = w;
+    }
+}
+
+// ---------------------------------------------------------------------------
+// k = 3, 4, 5 on the tensor cores, for matrices with no zero entry and entries within
+// 2^8 of the largest (then, as for two limbs, no range has to be checked in the
+// state). Fixed point of P bits in ND balanced digits of B bits, held as FP16
+// integers; a group's 2 2^k reals are one column of an mma.sync B operand, the
+// matrix (real 2 x 2 blocks) is A, and digit products of equal weight are summed
+// by the FP32 accumulators, exactly: |digit| <= 2^(B-1), so a sum of 2 2^k terms
+// and up to ND digit pairs stays within 2^24:
+//   k = 3, 4: 7 digits of 9 bits, 2^16 * 32 * 7 = 2^23.8
+//   k = 5:    8 digits of 8 bits, 2^14 * 64 * 8 = 2^23
+// Products of digits i, j (from the top) with i + j > ND are left out: below
+// 2^-65 of the full scale, random in sign.
+//
+// Why mma.sync: the matrix is 16 to 64 reals wide; a tcgen05 tile (128 rows)
+// would be mostly padding, and its operands would have to pass through shared
+// memory, where here a lane forms its own fragment registers: lane 4 c + q of
+// column c holds members q, q + 4, ... (re and im adjacent), and with re in rows
+// 0..7 and im in rows 8..15 of a tile it gets whole output amplitudes back.
+// Columns 2 q and 2 q + 1 are groups q and q + 4 of the warp's eight, so that a
+// store instruction covers 64 contiguous bytes per member.
+//
+// What bounds it: conversions to digits and back (about 110 instructions per
+// amplitude) and the MMAs, close to the time of the 32 bytes an amplitude moves.
+// ---------------------------------------------------------------------------
+constexpr int kFxtThreads = 256;
+
+template <int K> struct FxtCfg {
+    static constexpr int D = 1 << K, ND = K <= 4 ? 7 : 8, B = K <= 4 ? 9 : 8;
+    static constexpr int P = K <= 4 ? 61 : 62;
+#ifndef FXB
+#define FXB 2
+#endif
+    static constexpr int blocks = K == 3 ? 3 : K == 4 ? FXB : 1;
+    static constexpr int TM = D / 8;             // 16-row tiles of A, and 16-deep steps
+    static constexpr size_t smem = sizeof(uint4) * 32 * TM * TM * ND;
+};
+
+template <int K> struct Fxt {
+    long long m[1 << (2 * K)][2];   // round(2^(P - em) re, im)
+    double2 f[1 << (2 * K)];        // for groups out of range
+    int em;
+};
+
+// digit i (from the top) of the offset fixed-point numbers r, j as two FP16 integers
+template <int ND, int B>
+__device__ __forceinline__ uint32_t digits(uint64_t r, uint64_t j, int i) {
+    const int sh = B * (ND - 1 - i);
+    const uint32_t a = (uint32_t)(r >> sh), b = (uint32_t)(j >> sh);
+    constexpr uint32_t mask = ((1u << B) - 1u) * 0x00010001u;
+    uint32_t p = (__byte_perm(a, b, 0x5410) & mask) | 0x64006400u;        // 1024 + digit + 2^(B-1)
+    const uint32_t off = (0x6400u + (1u << (B - 1))) * 0x00010001u;
+    asm("sub.rn.f16x2 %0, %1, %2;" : "=r"(p) : "r"(p), "r"(off));
+    return p;
+}
+
+template <int ND, int B> __device__ __forceinline__ constexpr uint64_t digit_offset() {
+    uint64_t o = 0;
+    for (int i = 0; i < ND; ++i) o = (o << B) + (1ull << (B - 1));
+    return o;
+}
+
+__device__ __forceinline__ void mma16816(float (&c)[4], const uint4 &a, uint32_t b0, uint32_t b1) {
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+                 : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+                 : "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b0), "r"(b1));
+}
+
+template <int K>
+__global__ void __launch_bounds__(kFxtThreads, FxtCfg<K>::blocks)
+k_dense_fxt(double2 *__restrict__ sv, uint64_t n_groups, GroupGeom G, const __grid_constant__ Offs<K> O,
+            const Fxt<K> *__restrict__ Mg, const __grid_constant__ Fxt<(K <= 4 ? K : 1)> Mp) {
+    using Cfg = FxtCfg<K>;
+    constexpr int D = Cfg::D, ND = Cfg::ND, B = Cfg::B, P = Cfg::P, TM = Cfg::TM, NA = D / 4;
+    constexpr int NL = ND + 1;                        // levels: digit pairs i + j = 0 .. ND
+    constexpr uint64_t off = digit_offset<ND, B>();
+    extern __shared__ __align__(16) uint4 As[];       // [mt][ks][digit][lane]
+    const int lane = threadIdx.x & 31, q = lane & 3, c = lane >> 2;
+    const long long(*M)[2] = K <= 4 ? reinterpret_cast<const long long(*)[2]>(Mp.m) : Mg->m;
+    const double2 *Mf = K <= 4 ? reinterpret_cast<const double2 *>(Mp.f) : Mg->f;
+    const int em = K <= 4 ? Mp.em : Mg->em;
+    // A's fragments: lane 4 r + q holds rows r (re of member r) and r + 8 (its im),
+    // members q (registers x, y) and q + 4 (z, w) of the step
+    for (int i = threadIdx.x; i < TM * TM * 32; i += kFxtThreads) {
+        const int ln = i & 31, ks = (i >> 5) % TM, mt = (i >> 5) / TM;
+        const int row = mt * 8 + (ln >> 2), col = ks * 8 + (ln & 3);
+        const uint64_t r0 = off + (uint64_t)M[row * D + col][0], j0 = off + (uint64_t)M[row * D + col][1];
+        const uint64_t n0 = off - (uint64_t)M[row * D + col][1];
+        const uint64_t r1 = off + (uint64_t)M[row * D + col + 4][0], j1 = off + (uint64_t)M[row * D + col + 4][1];
+        const uint64_t n1 = off - (uint64_t)M[row * D + col + 4][1];
+#pragma unroll
+        for (int d = 0; d < ND; ++d)
+            As[((mt * TM + ks) * ND + d) * 32 + ln] = make_uint4(digits<ND, B>(r0, n0, d), digits<ND, B>(j0, r0, d),
+                                                                 digits<ND, B>(r1, n1, d), digits<ND, B>(j1, r1, d));
+    }
+    __syncthreads();
+    const int gcol = (c >> 1) + 4 * (c & 1);           // this lane's group of the eight as a B column
+    const uint64_t n_tiles = (n_groups + 7) / 8;
+    const uint64_t step = (uint64_t)gridDim.x * (kFxtThreads / 32);
+    uint64_t t = (uint64_t)blockIdx.x * (kFxtThreads / 32) + (threadIdx.x >> 5);
+    // a tile's amplitudes are loaded while the one before is computed
+    double2 v[NA];
+    uint64_t next = 0;
+    auto load = [&](uint64_t tile) {
+        const uint64_t g = tile * 8 + gcol;
+        next = insert_zeros(g < n_groups ? g : 0, G);
+#pragma unroll
+        for (int i = 0; i < NA; ++i) v[i] = sv[next + O.o[4 * i + q]];
+    };
+    if (t < n_tiles) load(t);
+    for (; t < n_tiles; t += step) {
+        const bool valid = t * 8 + gcol < n_groups;
+        const uint64_t base = next;
+        uint32_t b[NA][ND];
+        int E;
+        bool slow, zero;
+        {
+            int top = 0;
+            uint32_t any = 0;
+#pragma unroll
+            for (int i = 0; i < NA; ++i) {
+                const int hr = __double2hiint(v[i].x) & 0x7fffffff, hj = __double2hiint(v[i].y) & 0x7fffffff;
+                top = max(top, max(hr, hj));
+                any |= (uint32_t)__double2loint(v[i].x) | (uint32_t)__double2loint(v[i].y);
+            }
+#pragma unroll
+            for (int o = 1; o < 4; o <<= 1) {
+                top = max(top, __shfl_xor_sync(0xffffffffu, top, o));
+                any |= __shfl_xor_sync(0xffffffffu, any, o);
+            }
+            E = top >> 20;
+            zero = ((uint32_t)top | any) == 0;
+            slow = !zero && (unsigned)(E - kEMin) > (unsigned)(kEMax - kEMin);
+#pragma unroll
+            for (int i = 0; i < NA; ++i) {
+                auto fixed = [&](double w) {
+                    const int hi = __double2hiint(w);
+                    const uint64_t F = shr64(mant64(hi, __double2loint(w)), (uint32_t)(64 - P + E - ((hi >> 20) & 0x7ff)));
+                    return hi < 0 ? off - F : off + F;
+                };
+                const uint64_t fr = fixed(v[i].x), fj = fixed(v[i].y);
+#pragma unroll
+                for (int d = 0; d < ND; ++d) b[i][d] = digits<ND, B>(fr, fj, d);
+            }
+        }
+        bool store = valid && !slow && !zero;
+        if (__any_sync(0xffffffffu, slow)) {
+            // a group outside the exponent range: lane q computes rows q NA .. q NA + NA - 1 in FP64
+            double2 acc[NA];
+#pragma unroll
+            for (int j = 0; j < NA; ++j) acc[j] = make_double2(0.0, 0.0);
+            if (slow) {
+#pragma unroll 1
+                for (int l = 0; l < D; ++l) {
+                    const double2 w = sv[base + O.o[l]];
+#pragma unroll
+                    for (int j = 0; j < NA; ++j) cmad(acc[j], Mf[(q * NA + j) * D + l], w);
+                }
+            }
+            __syncwarp();                               // every lane has read its group before any writes it
+            if (slow && valid) {
+#pragma unroll
+                for (int j = 0; j < NA; ++j) sv[base + O.o[q * NA + j]] = acc[j];
+            }
+        }
+        if (t + step < n_tiles) load(t + step);
+        // what the output lanes need of columns 2 q and 2 q + 1
+        uint64_t ob[2];
+        int sc[2];
+        bool st[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int from = 4 * (2 * q + h);
+            ob[h] = __shfl_sync(0xffffffffu, base, from);
+            sc[h] = __shfl_sync(0xffffffffu, E, from) - 1022 + em - 2 * P + B * (ND - 2);
+            st[h] = __shfl_sync(0xffffffffu, (int)store, from) != 0;
+        }
+#pragma unroll 1
+        for (int mt = 0; mt < TM; ++mt) {
+            float a[NL][4];
+#pragma unroll
+            for (int p = 0; p < NL; ++p)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) a[p][e] = 0.f;
+#pragma unroll
+            for (int ks = 0; ks < TM; ++ks) {
+#pragma unroll
+                for (int i = 0; i < ND; ++i) {
+                    const uint4 f = As[((mt * TM + ks) * ND + i) * 32 + lane];
+#pragma unroll
+                    for (int j = 0; j < ND && i + j < NL; ++j) mma16816(a[i + j], f, b[2 * ks][j], b[2 * ks + 1][j]);
+                }
+            }
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                auto out = [&](int e) {
+                    int w[NL];
+#pragma unroll
+                    for (int p = 0; p < NL; ++p) w[p] = __float2int_rn(a[p][e]);     // exact: |a| <= 2^24
+                    // level p weighs 2^(B (ND - p)) units of the last one; the sum is hi 2^S + lo
+                    constexpr int S = B * (NL - 4);
+                    const long long hi = (long long)(w[0] * (1 << B) + w[1]) * (1 << (2 * B)) + (long long)w[2] * (1 << B) + w[3];
+                    long long lo = (long long)w[4] * (1 << (2 * B)) + (long long)w[5] * (1 << B) + w[6];
+#pragma unroll
+                    for (int p = 7; p < NL; ++p) lo = lo * (1 << B) + w[p];
+                    // 62 bits of it are rounded to the double's 53 (the FP64 pipe, which also
+                    // converts, is the scarce one: two conversions and a fused multiply-add
+                    // per real kept it 75 % busy)
+                    const int h1 = (int)(hi >> 32);
+                    const int cut = max(0, S + 2 - __clz(h1 ^ (h1 >> 31)));
+                    return scaled(__ll2double_rn((hi << (S - cut)) + (lo >> cut)), sc[h] + cut);
+                };
+                const double2 w = make_double2(out(h), out(2 + h));
+                if (st[h]) sv[ob[h] + O.o[mt * 8 + c]] = w;
+            }
+        }
     }
 }
 
@@ -412,8 +686,49 @@ cudaError_t run_fx3(const LaunchCtx &L, void *sv, uint64_t n_groups, const Group
         }
         M.f[i] = make_double2(mat[2 * i], mat[2 * i + 1]);
     }
-    k_dense_fx3<K><<<(unsigned)((n_groups + kThreads - 1) / kThreads), kThreads, 0, L.stream>>>(
+    constexpr int S = K >= 4 ? 2 : 1;
+    k_dense_fx3<K, S><<<(unsigned)((n_groups * S + kFx3Threads - 1) / kFx3Threads), kFx3Threads, 0, L.stream>>>(
         reinterpret_cast<double2 *>(sv), n_groups, G, O, M);
+    ++*L.launches;
+    return cudaGetLastError();
+}
+
+template <int K>
+cudaError_t run_fxt(const LaunchCtx &L, void *sv, uint64_t n_groups, const GroupGeom &G, const int *tpos,
+                    const double *mat, int em, void *d_mat) {
+    using Cfg = FxtCfg<K>;
+    Offs<K> O;
+    offsets<K>(tpos, O);
+    auto fill = [&](auto &M) {
+        M.em = em;
+        for (int i = 0; i < (1 << (2 * K)); ++i) {
+            for (int c = 0; c < 2; ++c) M.m[i][c] = (long long)to_fixed(mat[2 * i + c], em, Cfg::P);
+            M.f[i] = make_double2(mat[2 * i], mat[2 * i + 1]);
+        }
+    };
+    auto kern = k_dense_fxt<K>;
+    cudaError_t e = cudaSuccess;
+    if constexpr (Cfg::smem > 48 * 1024) {
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::smem);
+        if (e != cudaSuccess) return e;
+    }
+    constexpr uint64_t groups_per_block = 8 * (kFxtThreads / 32);
+    uint64_t grid = (n_groups + groups_per_block - 1) / groups_per_block;
+    const uint64_t most = (uint64_t)L.num_sms * Cfg::blocks;
+    if (grid > most) grid = most;
+    if constexpr (K <= 4) {
+        Fxt<K> M;
+        fill(M);
+        kern<<<(unsigned)grid, kFxtThreads, Cfg::smem, L.stream>>>(reinterpret_cast<double2 *>(sv), n_groups, G, O, nullptr,
+                                                                  M);
+    } else {
+        std::vector<Fxt<K>> hm(1);
+        fill(hm[0]);
+        e = cudaMemcpyAsync(d_mat, hm.data(), sizeof(Fxt<K>), cudaMemcpyHostToDevice, L.stream);
+        if (e != cudaSuccess) return e;
+        kern<<<(unsigned)grid, kFxtThreads, Cfg::smem, L.stream>>>(reinterpret_cast<double2 *>(sv), n_groups, G, O,
+                                                                  reinterpret_cast<const Fxt<K> *>(d_mat), Fxt<1>{});
+    }
     ++*L.launches;
     return cudaGetLastError();
 }
@@ -421,8 +736,8 @@ cudaError_t run_fx3(const LaunchCtx &L, void *sv, uint64_t n_groups, const Group
 }  // namespace
 
 bool try_dense_fx(const LaunchCtx &L, void *sv, int n, const GroupGeom &G, const int *tpos, int k, const double *mat,
-                  cudaError_t &e) {
-    if (k > 4) return false;
+                  void *d_mat, cudaError_t &e) {
+    if (k > 5) return false;
     const MatRange r = range_of(mat, 1 << (2 * k));
     if (!r.finite || r.em < -100 || r.em > 100) return false;
     const uint64_t n_groups = 1ull << (n - G.ns);
@@ -430,7 +745,13 @@ bool try_dense_fx(const LaunchCtx &L, void *sv, int n, const GroupGeom &G, const
         e = k == 1 ? run_fx2<1>(L, sv, n_groups, G, tpos, mat, r.em) : run_fx2<2>(L, sv, n_groups, G, tpos, mat, r.em);
         return true;
     }
-    if (r.dm > 16) return false;
+    if (k >= 3 && !r.zeros && r.dm <= (k == 5 ? 11 : 8)) {
+        e = k == 3   ? run_fxt<3>(L, sv, n_groups, G, tpos, mat, r.em, d_mat)
+            : k == 4 ? run_fxt<4>(L, sv, n_groups, G, tpos, mat, r.em, d_mat)
+                     : run_fxt<5>(L, sv, n_groups, G, tpos, mat, r.em, d_mat);
+        return true;
+    }
+    if (k > 4 || r.dm > 16) return false;
     switch (k) {
     case 1: e = run_fx3<1>(L, sv, n_groups, G, tpos, mat, r); break;
     case 2: e = run_fx3<2>(L, sv, n_groups, G, tpos, mat, r); break;

@@ -771,7 +771,7 @@ cudaError_t dense_any(const LaunchCtx &L, void *sv, int n, const GroupGeom &G, c
                       const double *mat, void *d_mat) {
     if constexpr (std::is_same<R, double>::value) {
         cudaError_t e;
-        if (try_dense_fx(L, sv, n, G, tpos, k, mat, e)) return e;
+        if (try_dense_fx(L, sv, n, G, tpos, k, mat, d_mat, e)) return e;
     }
     switch (k) {
     case 1: return dense_reg<R, 1>(L, sv, n, G, tpos, mat);

@@ -44,7 +44,7 @@ cudaError_t launch_dense(const LaunchCtx &L, sv_dtype_t dt, void *sv, int n, con
 // The same on a complex128 state in block fixed point (k_dense_fx.cu); false, with
 // nothing launched, where the matrix is outside the range it is as exact as FP64 for.
 bool try_dense_fx(const LaunchCtx &L, void *sv, int n, const GroupGeom &G, const int *tpos, int k, const double *mat,
-                  cudaError_t &e);
+                  void *d_mat, cudaError_t &e);
 // Diagonal d[j] on targets (any order; j's bit t is targets[t]) where controls hold, k = 0..6.
 cudaError_t launch_diag(const LaunchCtx &L, sv_dtype_t dt, void *sv, int n, const GroupGeom &Gctl,
                         const int *tpos, int k, const double *diag);

@@ -67,7 +67,8 @@ def states(n, rng):
     yield "basis", basis
 
 
-@pytest.mark.parametrize("targets", [(0,), (3,), (0, 1), (5, 2), (0, 4, 7), (8, 1, 3), (0, 1, 2, 3), (7, 3, 8, 5)])
+@pytest.mark.parametrize("targets", [(0,), (3,), (0, 1), (5, 2), (0, 4, 7), (8, 1, 3), (0, 1, 2, 3), (7, 3, 8, 5),
+                                     (0, 1, 2, 3, 4), (8, 2, 6, 3, 5)])
 def test_dense_matches_extended_precision(targets):
     rng = gen.rng_for(7 + len(targets))
     k = len(targets)
@@ -76,21 +77,26 @@ def test_dense_matches_extended_precision(targets):
     sparse = m.copy()
     sparse[rng.random(m.shape) < 0.3] = 0
     sparse[0, 0], sparse[0, -1] = 1, 0.5
-    for matrix in (m, near_identity, sparse, 1e30 * m, np.full(m.shape, -1.0 + 1.0j), m.real + 0j):
+    level = np.exp(2j * np.pi * rng.random(m.shape))   # every entry as large as the largest: full sums
+    edge = level.copy()
+    edge[0, 1], edge[-1, 0] = 2.0 ** -5 * (1 + 1j), 1e-3
+    for matrix in (m, level, edge, near_identity, sparse, 1e30 * m, np.full(m.shape, -1.0 + 1.0j), m.real + 0j):
         for _, v in states(9, rng):
             with np.errstate(all="ignore"):
                 check(v.astype(np.complex128), targets, matrix.astype(np.complex128))
 
 
 @pytest.mark.parametrize("n,targets,controls", [(1, (0,), ()), (2, (1, 0), ()), (3, (0, 2), (1,)), (4, (3, 0, 1, 2), ()),
-                                                (6, (4, 2, 5), (0, 3)), (13, (12,), (0,)), (13, (0, 6, 11, 12), (3,))])
+                                                (6, (4, 2, 5), (0, 3)), (13, (12,), (0,)), (13, (0, 6, 11, 12), (3,)), (4, (2, 0, 3), ()), (5, (1, 4, 2), ()),
+                                                (5, (0, 1, 2, 3, 4), ()), (7, (6, 0, 2, 5, 3), ()), (8, (1, 7, 4), (0, 2, 5)),
+                                                (15, (0, 9, 14, 3), ())])
 def test_dense_small_states_and_controls(n, targets, controls):
     rng = gen.rng_for(n)
     m = gen.random_gate_dense(rng, len(targets))
     check(gen.random_state(n, 3), targets, m, controls)
 
 
-@pytest.mark.parametrize("k", [1, 2, 3, 4])
+@pytest.mark.parametrize("k", [1, 2, 3, 4, 5])
 @pytest.mark.parametrize("bad", [np.inf, -np.inf, np.nan])
 def test_dense_nonfinite_groups_only(k, bad):
     """A non-finite amplitude spoils its own group, as in FP64, and no other."""
