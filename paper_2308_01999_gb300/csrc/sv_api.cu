@@ -9,7 +9,6 @@
 #include <cmath>
 #include <complex>
 #include <cstring>
-#include <map>
 #include <new>
 #include <vector>
 
@@ -572,8 +571,7 @@ sv_status_t sv_expectation_pauli(sv_handle_t h, const int *paulis, const int *si
                                  double *out) {
     if (!h || !out || n_sites < 0 || n_strings < 0 || ((!paulis || !sites) && n_sites > 0 && n_strings > 0))
         return SV_ERR_INVALID_ARGUMENT;
-    struct Str { uint64_t x, z; int ny; };
-    std::vector<Str> strs(n_strings);
+    std::vector<svk::PauliTerm> strs(n_strings);
     for (int s = 0; s < n_strings; ++s) {
         uint64_t x = 0, z = 0, seen = 0;
         int ny = 0;
@@ -602,44 +600,16 @@ sv_status_t sv_expectation_pauli(sv_handle_t h, const int *paulis, const int *si
             out[s] = strs[s].z ? h->h_results[__builtin_ctzll(strs[s].z)] : h->h_results[h->n];
         return SV_OK;
     }
-    // strings with the same X/Y mask share a pass over the state
-    std::map<uint64_t, std::vector<int>> by_x;
-    for (int s = 0; s < n_strings; ++s) by_x[strs[s].x].push_back(s);
-    std::vector<int> slot_of;   // result slot -> string
-    const svk::LaunchCtx L = lctx(h);
-    auto flush = [&]() -> sv_status_t {
-        if (slot_of.empty()) return SV_OK;
-        sv_status_t st = sync_results(h, (int)slot_of.size());
+    for (int s = 0; s < n_strings; s += h->max_results) {
+        const int m = std::min(n_strings - s, h->max_results);
+        if (svk::launch_pauli(lctx(h), h->dt, h->sv, h->n, strs.data() + s, m, h->d_partials, h->max_partial_blocks * 8,
+                              h->d_results) != cudaSuccess)
+            return SV_ERR_CUDA;
+        sv_status_t st = sync_results(h, m);
         if (st != SV_OK) return st;
-        for (size_t i = 0; i < slot_of.size(); ++i) out[slot_of[i]] = h->h_results[i];
-        slot_of.clear();
-        return SV_OK;
-    };
-    for (auto &kv : by_x) {
-        const std::vector<int> &ids = kv.second;
-        for (size_t b = 0; b < ids.size(); b += svk::kPauliMaxS) {
-            if ((int)slot_of.size() + svk::kPauliMaxS > h->max_results) {
-                sv_status_t st = flush();
-                if (st != SV_OK) return st;
-            }
-            svk::PauliPass P{};
-            P.S = (int)std::min<size_t>(svk::kPauliMaxS, ids.size() - b);
-            P.x = kv.first;
-            for (int i = 0; i < P.S; ++i) {
-                const Str &st = strs[ids[b + i]];
-                P.z[i] = st.z;
-                // Re(i^{nY} s w): +Re w, -Im w, -Re w, +Im w for nY = 0, 1, 2, 3 (mod 4)
-                const int r = st.ny & 3;
-                P.use_im[i] = r & 1;
-                P.sign[i] = (r == 1 || r == 2) ? -1.0 : 1.0;
-            }
-            cudaError_t e = svk::launch_pauli(L, h->dt, h->sv, h->n, P, h->d_partials, h->max_partial_blocks,
-                                              h->d_results + slot_of.size());
-            if (e != cudaSuccess) return SV_ERR_CUDA;
-            for (int i = 0; i < P.S; ++i) slot_of.push_back(ids[b + i]);
-        }
+        std::copy(h->h_results, h->h_results + m, out + s);
     }
-    return flush();
+    return SV_OK;
 }
 
 sv_status_t sv_apply_pauli_rotation(sv_handle_t h, double theta, const int *paulis, const int *sites, int n_sites) {

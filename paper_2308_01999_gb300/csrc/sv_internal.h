@@ -59,18 +59,16 @@ cudaError_t launch_swap(const LaunchCtx &L, sv_dtype_t dt, void *sv, int n, cons
 cudaError_t launch_pauli_rotation(const LaunchCtx &L, sv_dtype_t dt, void *sv, int n, uint64_t x, uint64_t z, int ny,
                                   double theta);
 
-// ---- reductions (k_reduce.cu) ----
-struct PauliPass {
-    int S;              // strings in this pass (1..8)
-    uint64_t x;         // common X|Y mask
-    uint64_t z[8];      // Z|Y mask per string
-    int use_im[8];      // take Im(w) instead of Re(w) (odd number of Y)
-    double sign[8];     // +1 / -1 from i^{nY}
+// ---- Pauli strings (k_pauli.cu) ----
+struct PauliTerm {
+    uint64_t x, z;      // X|Y and Z|Y masks
+    int ny;             // number of Y
 };
-constexpr int kPauliMaxS = 8;
-// Writes S doubles at d_out (device).
-cudaError_t launch_pauli(const LaunchCtx &L, sv_dtype_t dt, const void *sv, int n, const PauliPass &P,
-                         double *d_partials, int max_partial_blocks, double *d_out);
+// d_out[i] = <psi|terms[i]|psi> (device). d_partials: n_partials doubles of workspace, at least 16.
+cudaError_t launch_pauli(const LaunchCtx &L, sv_dtype_t dt, const void *sv, int n, const PauliTerm *terms, int count,
+                         double *d_partials, int n_partials, double *d_out);
+
+// ---- reductions (k_reduce.cu) ----
 // d_out[0] = sum over even parity of mask, d_out[1] = odd.
 cudaError_t launch_parity(const LaunchCtx &L, sv_dtype_t dt, const void *sv, int n, uint64_t mask,
                           double *d_partials, int max_partial_blocks, double *d_out);

@@ -22,9 +22,10 @@
 // before it is copied out. Calls whose work overlaps on the GPU (other streams,
 // other host threads) race on the array; the caller must order them.
 //
-// The kernels are the ones sv_expectation_pauli uses (k_reduce.cu), launched on
+// The kernels are the ones sv_expectation_pauli uses (k_pauli.cu), launched on
 // the caller's stream with the scratch address in place of the workspace.
 #include <mutex>
+#include <vector>
 
 #include "sv_internal.h"
 
@@ -111,30 +112,12 @@ extern "C" SV_API sv_status_t sv_expectation_pauli_noalloc(int n_qubits, sv_dtyp
     double *results = ds->addr + kPartialBlocks * 8;
     uint64_t launches = 0;
     const svk::LaunchCtx L{reinterpret_cast<cudaStream_t>(stream), ds->num_sms, &launches};
-    // one pass per run of at most 8 consecutive strings that share an X/Y mask;
-    // results land in string order
-    int s = 0;
-    while (s < n_strings) {
-        svk::PauliPass P{};
-        uint64_t x0, z;
-        int ny;
-        string_masks(paulis, sites, n_sites, s, n_qubits, x0, z, ny);
-        P.x = x0;
-        P.S = 0;
-        while (s + P.S < n_strings && P.S < svk::kPauliMaxS) {
-            uint64_t x;
-            string_masks(paulis, sites, n_sites, s + P.S, n_qubits, x, z, ny);
-            if (x != x0) break;
-            const int r = ny & 3;   // i^{nY}: +Re, -Im, -Re, +Im
-            P.z[P.S] = z;
-            P.use_im[P.S] = r & 1;
-            P.sign[P.S] = (r == 1 || r == 2) ? -1.0 : 1.0;
-            ++P.S;
-        }
-        if (svk::launch_pauli(L, dtype, d_state, n_qubits, P, partials, kPartialBlocks, results + s) != cudaSuccess)
-            return SV_ERR_CUDA;
-        s += P.S;
-    }
+    std::vector<svk::PauliTerm> terms(n_strings);
+    for (int s = 0; s < n_strings; ++s)
+        string_masks(paulis, sites, n_sites, s, n_qubits, terms[s].x, terms[s].z, terms[s].ny);
+    if (svk::launch_pauli(L, dtype, d_state, n_qubits, terms.data(), n_strings, partials, kPartialBlocks * 8, results) !=
+        cudaSuccess)
+        return SV_ERR_CUDA;
     if (cudaMemcpyAsync(out, results, sizeof(double) * n_strings, cudaMemcpyDeviceToHost, L.stream) != cudaSuccess)
         return SV_ERR_CUDA;
     return cudaStreamSynchronize(L.stream) == cudaSuccess ? SV_OK : SV_ERR_CUDA;
