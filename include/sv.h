@@ -187,6 +187,11 @@ typedef struct {
 SV_API sv_status_t sv_apply_fused_ex(sv_handle_t h, const sv_gate_t *gates, int n_gates,
                                      const sv_fusion_options_t *opt, int *n_fused_out);
 
+/* The gates in order, each applied as sv_apply_matrix applies it (no fusion),
+ * in one call. A gate that sv_apply_matrix would reject ends the call with its
+ * error; the gates before it have been enqueued. */
+SV_API sv_status_t sv_apply_circuit(sv_handle_t h, const sv_gate_t *gates, int n_gates);
+
 /* Host-only view of the fusion pass, for inspection and tests (no GPU needed).
  * Writes at most max_blocks blocks: block b acts on block_k[b] qubits
  * block_targets[6*b .. 6*b+k-1] (bit j of its matrix index is target j) with

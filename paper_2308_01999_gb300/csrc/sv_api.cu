@@ -10,6 +10,7 @@
 #include <complex>
 #include <cstring>
 #include <new>
+#include <utility>
 #include <vector>
 
 #include "sv_classify.h"
@@ -137,11 +138,7 @@ sv_status_t apply_gate(sv_ctx *h, Gate g, sv_precision_t prec) {
             return cuda_status(svk::launch_perm(L, h->dt, h->sv, h->n, G, g.t.data(), k, perm.data(), buf.data()));
         }
     }
-    buf.resize(2 * D * D);
-    for (int i = 0; i < D * D; ++i) {
-        buf[2 * i] = g.m[i].real();
-        buf[2 * i + 1] = g.m[i].imag();
-    }
+    const double *flat = reinterpret_cast<const double *>(g.m.data());   // (re, im) pairs
     if (prec != SV_PREC_NATIVE && h->dt == SV_C64 && k >= 5 && g.c.empty()) {
         // tensor-core path works on 6 targets; a 5-target block gains one identity
         // qubit, the highest one not in the block (low qubits stay free, which keeps
@@ -168,12 +165,12 @@ sv_status_t apply_gate(sv_ctx *h, Gate g, sv_precision_t prec) {
                 m6[2 * i + 1] = g6.m[i].imag();
             }
         } else {
-            m6 = buf;
+            m6.assign(flat, flat + 2 * D * D);
         }
         if (!svk::tc6_supported(h->n, t6.data())) return SV_ERR_NOT_SUPPORTED;
         return cuda_status(svk::launch_tc6(L, h->sv, h->n, t6.data(), m6.data(), prec, h->d_mat, h->d_err));
     }
-    return cuda_status(svk::launch_dense(L, h->dt, h->sv, h->n, G, g.t.data(), k, buf.data(), h->d_mat));
+    return cuda_status(svk::launch_dense(L, h->dt, h->sv, h->n, G, g.t.data(), k, flat, h->d_mat));
 }
 
 sv_status_t check_gate_args(const sv_ctx *h, const int *targets, int k, const int *controls, const int *cvals, int c,
@@ -418,6 +415,20 @@ sv_status_t sv_apply_matrix(sv_handle_t h, const int *targets, int n_targets, co
                       SV_PREC_NATIVE);
 }
 
+sv_status_t sv_apply_circuit(sv_handle_t h, const sv_gate_t *gates, int n_gates) {
+    if (!h || n_gates < 0 || (!gates && n_gates > 0)) return SV_ERR_INVALID_ARGUMENT;
+    DeviceGuard dg(h->device);
+    for (int i = 0; i < n_gates; ++i) {
+        const sv_gate_t &g = gates[i];
+        sv_status_t s = check_gate_args(h, g.targets, g.n_targets, g.controls, g.control_values, g.n_controls, g.matrix);
+        if (s != SV_OK) return s;
+        s = apply_gate(h, make_gate(g.targets, g.n_targets, g.controls, g.control_values, g.n_controls, g.matrix, 0),
+                       SV_PREC_NATIVE);
+        if (s != SV_OK) return s;
+    }
+    return SV_OK;
+}
+
 sv_status_t sv_swap_index_bits(sv_handle_t h, const int *bit_pairs, int n_pairs) {
     if (!h || !bit_pairs || n_pairs < 1 || n_pairs > 18) return SV_ERR_INVALID_ARGUMENT;
     int a[18], b[18];
@@ -543,19 +554,19 @@ sv_status_t sv_apply_fused_ex(sv_handle_t h, const sv_gate_t *gates, int n_gates
         s = sv_swap_index_bits(h, pairs.data(), npairs);
         if (s != SV_OK) return s;
     }
-    for (const svf::Item &it : items) {
+    for (svf::Item &it : items) {
         if (it.passthrough) {
             const sv_gate_t &g = gates[it.gate];
             Gate gg = make_gate(g.targets, g.n_targets, g.controls, g.control_values, g.n_controls, g.matrix, 0);
             for (int &q : gg.t) q = map[q];
             for (int &q : gg.c) q = map[q];
-            s = apply_gate(h, gg, prec);
+            s = apply_gate(h, std::move(gg), prec);
         } else {
             Gate g;
             g.t = it.qubits;
             for (int &q : g.t) q = map[q];
-            g.m = it.m;
-            s = apply_gate(h, g, prec);
+            g.m = std::move(it.m);
+            s = apply_gate(h, std::move(g), prec);
         }
         if (s != SV_OK) return s;
     }

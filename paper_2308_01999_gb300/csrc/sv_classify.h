@@ -81,15 +81,13 @@ inline void sort_targets(Gate &g) {
     bool ident = true;
     for (int i = 0; i < k; ++i) ident &= sigma[i] == i;
     if (ident) return;
-    auto old_index = [&](int rn) {
-        int ro = 0;
+    std::vector<int> old_index(D, 0);
+    for (int r = 0; r < D; ++r)
         for (int i = 0; i < k; ++i)
-            if ((rn >> i) & 1) ro |= 1 << sigma[i];
-        return ro;
-    };
+            if ((r >> i) & 1) old_index[r] |= 1 << sigma[i];
     std::vector<cd> m2(D * D);
     for (int r = 0; r < D; ++r)
-        for (int c = 0; c < D; ++c) m2[r * D + c] = g.m[old_index(r) * D + old_index(c)];
+        for (int c = 0; c < D; ++c) m2[r * D + c] = g.m[old_index[r] * D + old_index[c]];
     std::vector<int> t2(k);
     for (int i = 0; i < k; ++i) t2[i] = g.t[sigma[i]];
     g.t.swap(t2);

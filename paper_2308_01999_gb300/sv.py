@@ -11,6 +11,7 @@ missing.
 from __future__ import annotations
 
 import ctypes as C
+import itertools
 import os
 from dataclasses import dataclass
 
@@ -20,7 +21,7 @@ __all__ = [
     "SvError", "lib", "sv_create", "sv_destroy", "sv_set_stream", "sv_set_state_pointer", "sv_set_state",
     "sv_set_basis_state", "sv_copy_from_host", "sv_copy_to_host", "sv_copy_from_host_async",
     "sv_copy_to_host_async", "sv_apply_matrix",
-    "sv_apply_fused", "sv_fuse_plan", "sv_expectation_pauli", "sv_measure_probs", "sv_collapse",
+    "sv_apply_circuit", "sv_apply_fused", "sv_fuse_plan", "sv_expectation_pauli", "sv_measure_probs", "sv_collapse",
     "sv_measure", "sv_norm2", "sv_check_device_status", "sv_launch_count", "sv_status_string",
     "SV_C64", "SV_C128", "SV_PREC_NATIVE", "SV_PREC_TF32", "SV_PREC_SPLIT_BF16", "StateVector",
     "EXPORTED",
@@ -45,7 +46,7 @@ EXPORTED = [
     "sv_batch_results", "sv_swap_index_bits", "sv_apply_pauli_rotation", "sv_sample",
     "sv_check_bounded_wait", "sv_apply_fused_ex", "sv_fuse_plan_ex", "sv_copy_from_host_async",
     "sv_copy_to_host_async", "sv_batch_compile_ex", "sv_set_state", "sv_pool_create", "sv_pool_destroy",
-    "sv_pool_alloc", "sv_pool_free", "sv_pool_stats",
+    "sv_pool_alloc", "sv_pool_free", "sv_pool_stats", "sv_apply_circuit",
 ]
 
 
@@ -84,6 +85,7 @@ def lib():
             "sv_copy_from_host": [_VP, _VP], "sv_copy_to_host": [_VP, _VP],
             "sv_copy_from_host_async": [_VP, _VP], "sv_copy_to_host_async": [_VP, _VP],
             "sv_apply_matrix": [_VP, _I, C.c_int, _I, _I, C.c_int, _D, C.c_int],
+            "sv_apply_circuit": [_VP, C.POINTER(sv_gate_t), C.c_int],
             "sv_apply_fused": [_VP, C.POINTER(sv_gate_t), C.c_int, C.c_int, C.c_int, _I],
             "sv_fuse_plan": [C.POINTER(sv_gate_t), C.c_int, C.c_int, C.c_int, C.c_int, _I, _I, _I, _D],
             "sv_expectation_pauli": [_VP, _I, _I, C.c_int, C.c_int, _D],
@@ -199,23 +201,16 @@ def sv_apply_matrix(h: int, targets, matrix, controls=(), control_values=None, a
            "sv_apply_matrix")
 
 
-def _gate_array(gates):
-    arr = (sv_gate_t * max(1, len(gates)))()
-    keep = []
-    for i, g in enumerate(gates):
-        m, mp = _cmat(g.matrix)
-        keep.append(m)
-        s = arr[i]
-        s.n_targets = len(g.targets)
-        for j, q in enumerate(g.targets):
-            s.targets[j] = int(q)
-        s.n_controls = len(g.controls)
-        cv = tuple(g.control_values) if g.control_values else (1,) * len(g.controls)
-        for j, q in enumerate(g.controls):
-            s.controls[j] = int(q)
-            s.control_values[j] = int(cv[j])
-        s.matrix = mp
-    return arr, keep
+def _gate_array(gates, square: bool = False):
+    """``gates`` as an sv_gate_t pointer, and what has to outlive it."""
+    rec, buf = pack_gates(gates, square)
+    return C.cast(rec.ctypes.data, C.POINTER(sv_gate_t)), (rec, buf)
+
+
+def sv_apply_circuit(h: int, gates):
+    """Apply ``gates`` (objects with targets/matrix/controls/control_values) one by one, in one call."""
+    arr, _keep = _gate_array(gates, square=True)
+    _check(lib().sv_apply_circuit(_VP(h), arr, len(gates)), "sv_apply_circuit")
 
 
 def sv_apply_fused(h: int, gates, max_fused_qubits: int, prec: int = SV_PREC_NATIVE) -> int:
@@ -405,8 +400,14 @@ class StateVector:
         sv_apply_matrix(self.handle, g.targets, g.matrix, g.controls, g.control_values or None, adjoint)
 
     def apply_circuit(self, gates):
-        for g in gates:
-            self.apply_gate(g)
+        gates = list(gates)
+        try:
+            arr, _keep = _gate_array(gates, square=True)
+        except (TypeError, ValueError, IndexError, AttributeError):
+            for g in gates:         # a gate that cannot be packed: the ones before it still apply
+                self.apply_gate(g)
+            return
+        _check(lib().sv_apply_circuit(_VP(self.handle), arr, len(gates)), "sv_apply_circuit")
 
     def apply_fused(self, gates, max_fused_qubits: int, prec: int = SV_PREC_NATIVE,
                     max_fused_diagonal_qubits: int = 0) -> int:
@@ -465,37 +466,50 @@ ITEM_DTYPE = np.dtype([("n_qubits", "<i4"), ("gate_begin", "<i4"), ("n_gates", "
                        ("n_strings", "<i4"), ("out_begin", "<i4"), ("state_offset", "<u8")])
 
 
-def pack_gates(gates):
+def pack_gates(gates, square: bool = False):
     """sv_gate_t records for `gates` (a numpy structured array with the C layout)
     and the complex128 buffer their matrix pointers point into (keep both alive).
-    Gates are grouped by target and control count so that each group fills its
-    fields with one array assignment."""
+    Gates are grouped by target and control count, so that each group fills its
+    fields and its part of the buffer with one array operation. With `square`,
+    a matrix whose shape does not match its targets is a ValueError."""
     assert C.sizeof(sv_gate_t) == GATE_DTYPE.itemsize
     ng = len(gates)
     rec = np.zeros(ng, dtype=GATE_DTYPE)
     if ng == 0:
         return rec, np.empty(1, dtype=np.complex128)
-    mats = [np.asarray(g.matrix, dtype=np.complex128).reshape(-1) for g in gates]
-    sizes = np.fromiter((m.size for m in mats), dtype=np.int64, count=ng)
-    buf = np.concatenate(mats)
-    offs = np.zeros(ng, dtype=np.int64)
-    np.cumsum(sizes[:-1], out=offs[1:])
-    rec["matrix"] = np.uint64(buf.ctypes.data) + 16 * offs.astype(np.uint64)
-    kt = np.fromiter((len(g.targets) for g in gates), dtype=np.int32, count=ng)
-    kc = np.fromiter((len(g.controls) for g in gates), dtype=np.int32, count=ng)
-    rec["n_targets"] = kt
-    rec["n_controls"] = kc
-    for k in np.unique(kt):
-        idx = np.nonzero(kt == k)[0]
-        rec["targets"][idx, :k] = np.array([gates[i].targets for i in idx], dtype=np.int32).reshape(-1, k)
-    for c in np.unique(kc):
-        if c == 0:
-            continue
-        idx = np.nonzero(kc == c)[0]
-        rec["controls"][idx, :c] = np.array([gates[i].controls for i in idx], dtype=np.int32).reshape(-1, c)
-        rec["control_values"][idx, :c] = np.array(
-            [gates[i].control_values if gates[i].control_values else (1,) * c for i in idx],
-            dtype=np.int32).reshape(-1, c)
+    targets = [g.targets for g in gates]
+    controls = [g.controls for g in gates]
+    matrices = [g.matrix for g in gates]
+
+    def table(rows, width):
+        return np.fromiter(itertools.chain.from_iterable(rows), np.int32).reshape(len(rows), width)
+
+    groups = {}
+    for i, key in enumerate(zip(map(len, targets), map(len, controls))):
+        groups.setdefault(key, []).append(i)
+    buf = np.empty(sum(len(members) << (2 * k) for (k, _), members in groups.items()), dtype=np.complex128)
+    at = 0
+    for (k, c), members in groups.items():
+        if k > SV_MAX_TARGETS or c > SV_MAX_CONTROLS:
+            raise IndexError("too many targets or controls")
+        idx = slice(None) if len(groups) == 1 else np.array(members)
+        n, d = len(members), 1 << k
+        mats = [matrices[i] for i in members]
+        if {getattr(m, "shape", None) for m in mats} != {(d, d)}:
+            mats = [np.asarray(m, dtype=np.complex128) for m in mats]
+            if square and any(m.shape != (d, d) for m in mats):
+                raise ValueError("matrix shape does not match the number of targets")
+            mats = [m.reshape(-1)[:d * d].reshape(d, d) for m in mats]
+        np.concatenate(mats, out=buf[at:at + n * d * d].reshape(n * d, d), casting="unsafe")
+        rec["matrix"][idx] = buf.ctypes.data + 16 * (at + d * d * np.arange(n, dtype=np.uint64))
+        at += n * d * d
+        rec["n_targets"][idx] = k
+        rec["n_controls"][idx] = c
+        if k:
+            rec["targets"][idx, :k] = table([targets[i] for i in members], k)
+        if c:
+            rec["controls"][idx, :c] = table([controls[i] for i in members], c)
+            rec["control_values"][idx, :c] = table([gates[i].control_values or (1,) * c for i in members], c)
     return rec, buf
 
 
