@@ -1,6 +1,8 @@
 // k_common.cuh -- device helpers shared by the gate kernels.
 #pragma once
 
+#include <utility>
+
 #include "sv_internal.h"
 
 namespace svk {
@@ -37,6 +39,32 @@ __device__ __forceinline__ uint64_t insert_zeros(uint64_t g, const GroupGeom &G)
         g = ((g ^ lo) << 1) | lo;
     }
     return g | G.cset;
+}
+
+// Programmatic dependent launch: a gate kernel lets the next one start as soon as
+// all its blocks are running, and touches the state only after the one before
+// it has finished (and its writes are visible). On small states, where a kernel
+// takes about as long as its launch, the launch then overlaps the kernel before
+// (300 gates on 16 qubits: 4.1 us per gate launched plainly).
+__device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;"); }
+__device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// Launch a kernel that calls both. Every block has to reach wait_for_previous(),
+// or a later kernel could start before an earlier one is done.
+template <typename... P, typename... A>
+inline cudaError_t launch_dependent(void (*kern)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t stream,
+                                    A &&...args) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, std::forward<A>(args)...);
 }
 
 template <int K> struct Offs { uint64_t o[1 << K]; };

@@ -91,15 +91,18 @@ template <int K> struct Fx2 {
 };
 
 template <int K, int U>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kThreads, K == 1 ? 4 : 3)
 k_dense_fx2(double2 *__restrict__ sv, uint64_t n_groups, GroupGeom G, Offs<K> O, Fx2<K> M) {
     constexpr int D = 1 << K, P = Fx2<K>::P, PM = Fx2<K>::PM;
     const uint64_t u0 = (uint64_t)blockIdx.x * (kThreads * U) + threadIdx.x;
     double2 v[U][D];
     uint64_t base[U];
+    let_next_start();
+#pragma unroll
+    for (int u = 0; u < U; ++u) base[u] = insert_zeros(u0 + (uint64_t)u * kThreads, G);
+    wait_for_previous();
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-        base[u] = insert_zeros(u0 + (uint64_t)u * kThreads, G);
         if (u0 + (uint64_t)u * kThreads < n_groups) {
 #pragma unroll
             for (int j = 0; j < D; ++j) v[u][j] = sv[base[u] + O.o[j]];
@@ -230,6 +233,7 @@ k_dense_fx3(double2 *__restrict__ sv, uint64_t n_groups, GroupGeom G, const __gr
     constexpr int D = 1 << K, DL = D / S;
     constexpr int RS = (DL * 8 + (S > 1 ? 8 : 0)) * S;   // ints of a row; lanes' parts 8 banks apart
     __shared__ __align__(16) int Ms[D * RS];
+    let_next_start();
     for (int i = threadIdx.x; i < D * D * 6; i += kFx3Threads) {
         const int e = i / 6, j = e / D, l = e % D;
         Ms[j * RS + (l / DL) * (RS / S) + (l % DL) * 8 + i % 6] = M.m[e][i % 6];
@@ -240,6 +244,7 @@ k_dense_fx3(double2 *__restrict__ sv, uint64_t n_groups, GroupGeom G, const __gr
     const bool valid = g < n_groups;
     if (!valid) g = 0;                                  // whole warps take part in the exchanges; nothing is stored
     const uint64_t base = insert_zeros(g, G);
+    wait_for_previous();
     int x[2 * DL][3];
     int E;
     bool slow, zero;
@@ -448,6 +453,8 @@ k_dense_fxt(double2 *__restrict__ sv, uint64_t n_groups, GroupGeom G, const __gr
     const int lane = threadIdx.x & 31, q = lane & 3, c = lane >> 2;
     const long long(*M)[2] = K <= 4 ? reinterpret_cast<const long long(*)[2]>(Mp.m) : Mg->m;
     const double2 *Mf = K <= 4 ? reinterpret_cast<const double2 *>(Mp.f) : Mg->f;
+    let_next_start();
+    if constexpr (K > 4) wait_for_previous();          // the matrix is in the workspace
     const int em = K <= 4 ? Mp.em : Mg->em;
     // A's fragments: lane 4 r + q holds rows r (re of member r) and r + 8 (its im),
     // members q (registers x, y) and q + 4 (z, w) of the step
@@ -477,6 +484,7 @@ k_dense_fxt(double2 *__restrict__ sv, uint64_t n_groups, GroupGeom G, const __gr
 #pragma unroll
         for (int i = 0; i < NA; ++i) v[i] = sv[next + O.o[4 * i + q]];
     };
+    if constexpr (K <= 4) wait_for_previous();
     if (t < n_tiles) load(t);
     for (; t < n_tiles; t += step) {
         const bool valid = t * 8 + gcol < n_groups;
@@ -663,10 +671,9 @@ cudaError_t run_fx2(const LaunchCtx &L, void *sv, uint64_t n_groups, const Group
         M.f[i] = make_double2(mat[2 * i], mat[2 * i + 1]);
     }
     const uint64_t per = (uint64_t)kThreads * U;
-    k_dense_fx2<K, U><<<(unsigned)((n_groups + per - 1) / per), kThreads, 0, L.stream>>>(
-        reinterpret_cast<double2 *>(sv), n_groups, G, O, M);
     ++*L.launches;
-    return cudaGetLastError();
+    return launch_dependent(k_dense_fx2<K, U>, (unsigned)((n_groups + per - 1) / per), kThreads, 0, L.stream,
+                            reinterpret_cast<double2 *>(sv), n_groups, G, O, M);
 }
 
 template <int K>
@@ -687,10 +694,9 @@ cudaError_t run_fx3(const LaunchCtx &L, void *sv, uint64_t n_groups, const Group
         M.f[i] = make_double2(mat[2 * i], mat[2 * i + 1]);
     }
     constexpr int S = K >= 4 ? 2 : 1;
-    k_dense_fx3<K, S><<<(unsigned)((n_groups * S + kFx3Threads - 1) / kFx3Threads), kFx3Threads, 0, L.stream>>>(
-        reinterpret_cast<double2 *>(sv), n_groups, G, O, M);
     ++*L.launches;
-    return cudaGetLastError();
+    return launch_dependent(k_dense_fx3<K, S>, (unsigned)((n_groups * S + kFx3Threads - 1) / kFx3Threads), kFx3Threads,
+                            0, L.stream, reinterpret_cast<double2 *>(sv), n_groups, G, O, M);
 }
 
 template <int K>
@@ -716,21 +722,20 @@ cudaError_t run_fxt(const LaunchCtx &L, void *sv, uint64_t n_groups, const Group
     uint64_t grid = (n_groups + groups_per_block - 1) / groups_per_block;
     const uint64_t most = (uint64_t)L.num_sms * Cfg::blocks;
     if (grid > most) grid = most;
+    ++*L.launches;
+    double2 *psi = reinterpret_cast<double2 *>(sv);
     if constexpr (K <= 4) {
         Fxt<K> M;
         fill(M);
-        kern<<<(unsigned)grid, kFxtThreads, Cfg::smem, L.stream>>>(reinterpret_cast<double2 *>(sv), n_groups, G, O, nullptr,
-                                                                  M);
+        return launch_dependent(kern, (unsigned)grid, kFxtThreads, Cfg::smem, L.stream, psi, n_groups, G, O, nullptr, M);
     } else {
         std::vector<Fxt<K>> hm(1);
         fill(hm[0]);
         e = cudaMemcpyAsync(d_mat, hm.data(), sizeof(Fxt<K>), cudaMemcpyHostToDevice, L.stream);
         if (e != cudaSuccess) return e;
-        kern<<<(unsigned)grid, kFxtThreads, Cfg::smem, L.stream>>>(reinterpret_cast<double2 *>(sv), n_groups, G, O,
-                                                                  reinterpret_cast<const Fxt<K> *>(d_mat), Fxt<1>{});
+        return launch_dependent(kern, (unsigned)grid, kFxtThreads, Cfg::smem, L.stream, psi, n_groups, G, O,
+                                reinterpret_cast<const Fxt<K> *>(d_mat), Fxt<1>{});
     }
-    ++*L.launches;
-    return cudaGetLastError();
 }
 
 }  // namespace

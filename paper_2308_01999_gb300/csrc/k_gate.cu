@@ -56,10 +56,16 @@ k_dense(typename CT<R>::T *__restrict__ sv, uint64_t n_units, GroupGeom G, Offs<
     const uint64_t u0 = (uint64_t)blockIdx.x * (kThreads * U) + threadIdx.x;
     C v[U][D][E];
     uint64_t base[U];
+    let_next_start();
 #pragma unroll
     for (int u = 0; u < U; ++u) {
         const uint64_t unit = u0 + (uint64_t)u * kThreads;
         base[u] = insert_zeros(MODE == PAIR ? (unit << 1) : unit, G);
+    }
+    wait_for_previous();
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+        const uint64_t unit = u0 + (uint64_t)u * kThreads;
         if (unit < n_units) {
             if constexpr (MODE == PAIR) {
 #pragma unroll
@@ -208,8 +214,10 @@ k_dense_blk(float2 *__restrict__ sv, uint64_t n_sg, GroupGeom Ghi, LoOffs<KLO> O
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     float2 *buf = sm[warp];
     const uint64_t sgi = (uint64_t)blockIdx.x * (kThreads / 32) + warp;
-    if (sgi >= n_sg) return;                   // warp-uniform
+    let_next_start();
     const uint64_t base = insert_zeros(sgi << B, Ghi);
+    wait_for_previous();
+    if (sgi >= n_sg) return;                   // warp-uniform
     float4 v[PER];
 #pragma unroll
     for (int r = 0; r < PER; ++r) {
@@ -461,13 +469,16 @@ __global__ void __launch_bounds__(kThreads)
 k_diag(typename CT<R>::T *__restrict__ sv, uint64_t n_units, GroupGeom G, DiagP<R> P) {
     using C = typename CT<R>::T;
     const uint64_t u0 = (uint64_t)blockIdx.x * (kThreads * U) + threadIdx.x;
+    let_next_start();
     if constexpr (MODE == PAIR) {
         float4 f[U];
         uint64_t idx[U];
 #pragma unroll
+        for (int u = 0; u < U; ++u) idx[u] = insert_zeros((u0 + (uint64_t)u * kThreads) << 1, G);
+        wait_for_previous();
+#pragma unroll
         for (int u = 0; u < U; ++u) {
             const uint64_t unit = u0 + (uint64_t)u * kThreads;
-            idx[u] = insert_zeros(unit << 1, G);
             if (unit < n_units) f[u] = ld16(reinterpret_cast<const float2 *>(sv) + idx[u]);
         }
 #pragma unroll
@@ -481,9 +492,11 @@ k_diag(typename CT<R>::T *__restrict__ sv, uint64_t n_units, GroupGeom G, DiagP<
         C a[U];
         uint64_t idx[U];
 #pragma unroll
+        for (int u = 0; u < U; ++u) idx[u] = insert_zeros(u0 + (uint64_t)u * kThreads, G);
+        wait_for_previous();
+#pragma unroll
         for (int u = 0; u < U; ++u) {
             const uint64_t unit = u0 + (uint64_t)u * kThreads;
-            idx[u] = insert_zeros(unit, G);
             if (unit < n_units) a[u] = sv[idx[u]];
         }
 #pragma unroll
@@ -513,10 +526,16 @@ k_perm(typename CT<R>::T *__restrict__ sv, uint64_t n_units, GroupGeom G, PermP<
     const uint64_t u0 = (uint64_t)blockIdx.x * (kThreads * U) + threadIdx.x;
     C v[U][D][E];
     uint64_t base[U];
+    let_next_start();
 #pragma unroll
     for (int u = 0; u < U; ++u) {
         const uint64_t unit = u0 + (uint64_t)u * kThreads;
         base[u] = insert_zeros(MODE == PAIR ? (unit << 1) : unit, G);
+    }
+    wait_for_previous();
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+        const uint64_t unit = u0 + (uint64_t)u * kThreads;
         if (unit < n_units) {
 #pragma unroll
             for (int l = 0; l < D; ++l) {
@@ -566,19 +585,17 @@ template <typename R, int K, int MODE>
 cudaError_t run_dense_reg(const LaunchCtx &L, void *sv, uint64_t n_units, const GroupGeom &G, const Offs<K> &O,
                           const MatK<R, K> &M) {
     constexpr int U = dense_u<R, K, MODE>();
-    k_dense<R, K, MODE, U><<<grid_for(n_units, kThreads * U), kThreads, 0, L.stream>>>(
-        reinterpret_cast<typename CT<R>::T *>(sv), n_units, G, O, M);
     ++*L.launches;
-    return cudaGetLastError();
+    return launch_dependent(k_dense<R, K, MODE, U>, grid_for(n_units, kThreads * U), kThreads, 0, L.stream,
+                            reinterpret_cast<typename CT<R>::T *>(sv), n_units, G, O, M);
 }
 
 template <int K, int KLO>
 cudaError_t run_dense_blk(const LaunchCtx &L, void *sv, uint64_t n_sg, const GroupGeom &Ghi, const LoOffs<KLO> &Olo,
                           const Offs<K - KLO> &Ohi, const MatK<float, K> &M) {
-    k_dense_blk<K, KLO><<<grid_for(n_sg, kThreads / 32), kThreads, 0, L.stream>>>(reinterpret_cast<float2 *>(sv), n_sg,
-                                                                                   Ghi, Olo, Ohi, M);
     ++*L.launches;
-    return cudaGetLastError();
+    return launch_dependent(k_dense_blk<K, KLO>, grid_for(n_sg, kThreads / 32), kThreads, 0, L.stream,
+                            reinterpret_cast<float2 *>(sv), n_sg, Ghi, Olo, Ohi, M);
 }
 
 // The warp-staged kernel takes a dense gate on a complex64 state when qubit 1
@@ -801,19 +818,13 @@ cudaError_t diag_any(const LaunchCtx &L, void *sv, int n, const GroupGeom &Gc, c
     const uint64_t n_amps = 1ull << (n - Gc.ns);
     const bool bit0_ctl = Gc.ns > 0 && Gc.pos[0] == 0;
     constexpr int U = 4;
-    bool done = false;
-    if constexpr (sizeof(R) == 4) {
-        if (!bit0_ctl && n_amps >= 2) {
-            k_diag<R, PAIR, U><<<grid_for(n_amps / 2, kThreads * U), kThreads, 0, L.stream>>>(
-                reinterpret_cast<C *>(sv), n_amps / 2, Gc, P);
-            done = true;
-        }
-    }
-    if (!done)
-        k_diag<R, SCALAR, U><<<grid_for(n_amps, kThreads * U), kThreads, 0, L.stream>>>(
-            reinterpret_cast<C *>(sv), n_amps, Gc, P);
     ++*L.launches;
-    return cudaGetLastError();
+    if constexpr (sizeof(R) == 4)
+        if (!bit0_ctl && n_amps >= 2)
+            return launch_dependent(k_diag<R, PAIR, U>, grid_for(n_amps / 2, kThreads * U), kThreads, 0, L.stream,
+                                    reinterpret_cast<C *>(sv), n_amps / 2, Gc, P);
+    return launch_dependent(k_diag<R, SCALAR, U>, grid_for(n_amps, kThreads * U), kThreads, 0, L.stream,
+                            reinterpret_cast<C *>(sv), n_amps, Gc, P);
 }
 
 template <typename R, int K>
@@ -837,19 +848,13 @@ cudaError_t perm_k(const LaunchCtx &L, void *sv, int n, const GroupGeom &G, cons
     const uint64_t n_groups = 1ull << (n - G.ns);
     const bool bit0_special = G.ns > 0 && G.pos[0] == 0;
     constexpr int U = (K <= 2) ? 2 : 1;
-    bool done = false;
-    if constexpr (sizeof(R) == 4) {
-        if (!bit0_special && n_groups >= 2) {
-            k_perm<R, K, PAIR, U><<<grid_for(n_groups / 2, kThreads * U), kThreads, 0, L.stream>>>(
-                reinterpret_cast<C *>(sv), n_groups / 2, G, P);
-            done = true;
-        }
-    }
-    if (!done)
-        k_perm<R, K, SCALAR, U><<<grid_for(n_groups, kThreads * U), kThreads, 0, L.stream>>>(
-            reinterpret_cast<C *>(sv), n_groups, G, P);
     ++*L.launches;
-    return cudaGetLastError();
+    if constexpr (sizeof(R) == 4)
+        if (!bit0_special && n_groups >= 2)
+            return launch_dependent(k_perm<R, K, PAIR, U>, grid_for(n_groups / 2, kThreads * U), kThreads, 0, L.stream,
+                                    reinterpret_cast<C *>(sv), n_groups / 2, G, P);
+    return launch_dependent(k_perm<R, K, SCALAR, U>, grid_for(n_groups, kThreads * U), kThreads, 0, L.stream,
+                            reinterpret_cast<C *>(sv), n_groups, G, P);
 }
 
 template <typename R>
