@@ -49,6 +49,7 @@
 #include <vector>
 
 #include "sv_internal.h"
+#include "tc_common.cuh"
 
 namespace svk {
 namespace {
@@ -65,8 +66,6 @@ constexpr int kBStage = 64 * 1024;    // bytes of one B tile (either precision)
 constexpr int kTmemCols = 2 * kNT;    // two accumulators
 constexpr int kStgPitch = 17;         // floats per staged accumulator row (16 columns + 1 against bank conflicts)
 constexpr int kEpiStage = kEpiWarps * 32 * kStgPitch * 4;   // bytes of epilogue staging
-constexpr long long kWaitCycles = 4000000000ll;   // ~2 s at 2 GHz
-constexpr int kErrTimeout = 0x7c01;
 
 enum Prec { TF32 = 1, BF16 = 2 };
 
@@ -85,68 +84,11 @@ struct TcTab {
     uint64_t adr_lo[128], adr_hi[64];   // a's bits 0..6 / 7..12 -> amplitude offset
     uint16_t ij_lo[128], ij_hi[64];     // the same bits -> column i | member j << 7
 };
-constexpr int kErrSmemAlign = 0x7c02;
 
 // dynamic shared memory of k_tc6: operands, staging, control
 __host__ __device__ constexpr int tc_stage_off() { return kAImg + 2 * kBStage; }
 __host__ __device__ constexpr int tc_ctl_off() { return tc_stage_off() + kEpiStage; }
 __host__ __device__ constexpr int tc_smem_bytes() { return tc_ctl_off() + (int)sizeof(TcCtl); }
-
-__device__ __forceinline__ uint32_t smem_u32(const void *p) {
-    return static_cast<uint32_t>(__cvta_generic_to_shared(p));
-}
-
-__device__ __forceinline__ void mbar_init(uint32_t a, uint32_t count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(a), "r"(count) : "memory");
-}
-
-__device__ __forceinline__ void mbar_arrive(uint32_t a) {
-    asm volatile("{\n\t.reg .b64 st;\n\tmbarrier.arrive.shared::cta.b64 st, [%0];\n\t}" ::"r"(a) : "memory");
-}
-
-__device__ __forceinline__ bool mbar_try(uint32_t a, uint32_t parity) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(a), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-
-// Bounded wait: false on timeout or when another role has aborted.
-__device__ __forceinline__ bool mbar_wait(uint32_t a, uint32_t parity, volatile int *abort_flag, int *d_err,
-                                          long long budget = kWaitCycles) {
-    const long long t0 = clock64();
-    while (!mbar_try(a, parity)) {
-        if (*abort_flag) return false;
-        if (clock64() - t0 > budget) {
-            *abort_flag = 1;
-            atomicExch(d_err, kErrTimeout);
-            return false;
-        }
-    }
-    return true;
-}
-
-__device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-
-// Shared-memory matrix descriptor (tcgen05): start address, leading byte offset
-// (unused for swizzled K-major, set to 16 B), stride byte offset 1024 B (eight
-// 128-byte rows), descriptor version 1, 128-byte swizzle.
-__device__ __forceinline__ uint64_t sdesc(uint32_t addr) {
-    uint64_t d = 0;
-    d |= (uint64_t)((addr & 0x3FFFFu) >> 4);
-    d |= (uint64_t)(16u >> 4) << 16;
-    d |= (uint64_t)(1024u >> 4) << 32;
-    d |= 1ull << 46;
-    d |= 2ull << 61;
-    return d;
-}
 
 // Instruction descriptor: D = F32, A/B format (TF32 = 2, BF16 = 1), both K-major,
 // N = 128 (bits 17-22 hold N >> 3), M = 128 (bits 24-28 hold M >> 4).
@@ -172,39 +114,6 @@ __device__ __forceinline__ void mma(uint32_t d_tmem, uint64_t a, uint64_t b, uin
     }
 }
 
-__device__ __forceinline__ void mma_commit(uint32_t bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
-}
-
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
-    uint32_t r[32];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-        "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-        "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-          "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-          "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-        : "r"(taddr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-    for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
-}
-
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
-    uint32_t r[16];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-        "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-    for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
-}
-
 __device__ __forceinline__ uint32_t to_tf32(float x) {
     uint32_t r;
     asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
@@ -218,22 +127,6 @@ __device__ __forceinline__ void split_bf16(float a, float b, uint32_t &hi, uint3
     const __nv_bfloat162 l = __floats2bfloat162_rn(a - hf.x, b - hf.y);
     hi = *reinterpret_cast<const uint32_t *>(&h);
     lo = *reinterpret_cast<const uint32_t *>(&l);
-}
-
-struct TcGeom {
-    int pos[6];          // target positions, ascending
-    uint64_t off[64];    // member offsets
-    uint64_t n_cols;     // 2^(n-6)
-    uint64_t n_tiles;
-};
-
-__device__ __forceinline__ uint64_t col_base(uint64_t c, const TcGeom &G) {
-#pragma unroll
-    for (int i = 0; i < 6; ++i) {
-        const uint64_t lo = c & ((1ull << G.pos[i]) - 1ull);
-        c = ((c ^ lo) << 1) | lo;
-    }
-    return c;
 }
 
 // byte offset of the 16-byte chunk `chunk` (0..7 within the 128-byte row) of
@@ -507,15 +400,6 @@ constexpr int kGuard3 = 2048;              // unused bytes after the last stage
 constexpr int kSmem3 = kA3 + kStages3 * kB3 + kGuard3 + (int)sizeof(TcCtl3);
 static_assert(kSmem3 <= 227 * 1024, "dynamic shared memory of the raw-operand kernel exceeds the per-block limit");
 
-// byte offset of the 16-byte chunk holding floats 4c .. 4c+3 of member row l
-// (c = amplitude pair, 0..63) in a stage: atom (c / 8, l / 8); inside it rows of
-// 128 bytes (32 floats of one member) whose four 32-byte units are permuted by
-// the row index mod 4
-__device__ __forceinline__ uint32_t mn_chunk(int l, int c) {
-    return (uint32_t)((c >> 3) * 8192 + (l >> 3) * 1024 + (l & 7) * 128 + ((((c & 7) >> 1) ^ (l & 3)) << 5) +
-                      ((c & 1) << 4));
-}
-
 // MN-major operand descriptor: column atoms 8192 bytes apart (leading offset),
 // 8-row member groups `sbo` bytes apart, swizzle `mode` (1: 128 bytes with
 // 32-byte atomicity, 4: 64 bytes). Either reading of the two offsets stays
@@ -584,33 +468,6 @@ __device__ __forceinline__ void split_atom(uint32_t atom, int lane) {
                  : "memory");
     __syncwarp();
 }
-
-__device__ __forceinline__ void cp_async16(uint32_t dst, const void *src, uint32_t src_bytes) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(src_bytes) : "memory");
-}
-
-// Which chunk of the tile each copy (and store) moves is set by the host
-// (RawMap): with qubit 0 free a chunk is amplitudes (2p, 2p + 1) of member row l
-// (2 x 6 index bits: the member's bits sit at the target positions, the pair's at
-// non-target positions 1..6); with qubit 0 a target (T0) it is members 2m, 2m + 1
-// of one column c (5 member-pair bits at target positions 1..5, 7 column bits at
-// the non-target positions), landed in row 2m + (c & 1) of pair c / 2 and turned
-// into member rows by the convert stage. The index bits are ordered by the
-// address position they set (the three lowest lane bits chosen among the low
-// ones so that eight consecutive lanes hit eight different 16-byte bank groups
-// of shared memory); the five first vary across the lanes of a warp, the next
-// one across the two copy warps, the rest across a thread's copies.
-// Both the amplitude address and the operand offset (mn_chunk is linear over
-// XOR) are OR / XOR of per-bit contributions, so a thread combines one
-// per-thread and one per-copy table entry.
-struct RawMap {
-    uint64_t cthr_addr[64], cit_addr[64];   // copy: amplitude offset, thread part / copy part
-    uint32_t cthr_sm[64], cit_sm[64];       // copy: operand byte offset in a stage
-    uint32_t cthr_col[64], cit_col[64];     // copy: first column of the chunk (ragged tiles)
-    uint64_t sl_addr[32], sr_addr[16];      // store: lane part / iteration part (one epilogue warp)
-    uint32_t sl_sm[32], sr_sm[16];
-    uint32_t sl_col[32], sr_col[16];
-};
 
 // Copy and store orders: PLAIN and IL are fixed orders for qubit 0 free (PLAIN:
 // each instruction 32 consecutive amplitude pairs of one member; IL, lowest
@@ -957,27 +814,6 @@ uint32_t host_tf32(float x) {
     return u & 0xffffe000u;
 }
 
-uint16_t host_bf16(float x) {
-    // round to nearest even
-    uint32_t u;
-    std::memcpy(&u, &x, 4);
-    if ((u & 0x7f800000u) == 0x7f800000u) return (uint16_t)(u >> 16);
-    const uint32_t lsb = (u >> 16) & 1u;
-    u += 0x7fffu + lsb;
-    return (uint16_t)(u >> 16);
-}
-
-float bf16_to_float(uint16_t h) {
-    const uint32_t u = (uint32_t)h << 16;
-    float f;
-    std::memcpy(&f, &u, 4);
-    return f;
-}
-
-size_t host_sw128(int kb, int r, int chunk) {
-    return (size_t)kb * (128 * 128) + (size_t)(r >> 3) * 1024 + (size_t)(r & 7) * 128 + (size_t)((chunk ^ (r & 7)) << 4);
-}
-
 // A[2j+e][2l+f] from G (64x64 complex, row-major, interleaved doubles)
 double a_real(const double *g, int m, int k) {
     const int j = m >> 1, e = m & 1, l = k >> 1, f = k & 1;
@@ -1042,107 +878,6 @@ cudaError_t run_tc_raw(const LaunchCtx &L, float2 *sv, const TcGeom &G, const Ra
     return cudaGetLastError();
 }
 
-// operand byte offset of row l, amplitude pair c in a stage (the host twin of mn_chunk)
-uint32_t host_mn_chunk(int l, int c) {
-    return (uint32_t)((c >> 3) * 8192 + (l >> 3) * 1024 + (l & 7) * 128 + ((((c & 7) >> 1) ^ (l & 3)) << 5) +
-                      ((c & 1) << 4));
-}
-
-// The address-ordered chunk mapping of the raw-operand kernel for targets tpos on
-// an n-qubit state (see RawMap). Each index bit of a chunk has an amplitude
-// address bit, an operand offset and a column contribution; the bits are sorted
-// by address bit and dealt out to lanes first.
-RawMap build_raw_map(int n, const int *tpos, bool t0) {
-    std::vector<int> npos;                       // non-target positions, ascending; past n for tiny states
-    for (int q = 0, t = 0; (int)npos.size() < 8; ++q) {
-        if (t < 6 && q == tpos[t]) {
-            ++t;
-            continue;
-        }
-        npos.push_back(q);
-    }
-    struct Bit { int apos; uint64_t addr; uint32_t sm; uint32_t col; };
-    auto member_bit = [&](int i) {      // member index bit i (row bit i with qubit 0 free)
-        return Bit{tpos[i], 1ull << tpos[i], host_mn_chunk(1 << i, 0), 0u};
-    };
-    std::vector<Bit> copy, store;
-    if (!t0) {
-        for (int i = 0; i < 6; ++i)     // pair bit i: column bit i + 1
-            copy.push_back(Bit{npos[i + 1], 1ull << npos[i + 1], host_mn_chunk(0, 1 << i), 2u << i});
-        for (int i = 0; i < 6; ++i) copy.push_back(member_bit(i));
-        for (int i = 0; i < 5; ++i)
-            store.push_back(Bit{npos[i + 1], 1ull << npos[i + 1], host_mn_chunk(0, 1 << i), 2u << i});
-        for (int i = 0; i < 4; ++i) store.push_back(member_bit(i));
-    } else {
-        // member-pair bit i (member bit i + 1, row bit i + 1); column bit 0 selects the
-        // row of the pair, column bit i >= 1 is pair bit i - 1
-        auto pair_bit = [&](int i) {
-            return Bit{tpos[i + 1], 1ull << tpos[i + 1], host_mn_chunk(2 << i, 0), 0u};
-        };
-        auto col_bit = [&](int i) {
-            return Bit{npos[i], 1ull << npos[i], i == 0 ? host_mn_chunk(1, 0) : host_mn_chunk(0, 1 << (i - 1)), 1u << i};
-        };
-        for (int i = 0; i < 5; ++i) copy.push_back(pair_bit(i));
-        for (int i = 0; i < 7; ++i) copy.push_back(col_bit(i));
-        for (int i = 0; i < 3; ++i) store.push_back(pair_bit(i));
-        for (int i = 0; i < 6; ++i) store.push_back(col_bit(i));
-    }
-    // Address order, except that lanes 0-2 (the eight lanes of one shared-memory
-    // wavefront of 16-byte accesses) take the lowest bits whose operand offsets
-    // fall in independent 16-byte bank groups, so that those accesses never
-    // conflict; the other bits follow in address order.
-    auto order = [](std::vector<Bit> &bits) {
-        std::sort(bits.begin(), bits.end(), [](const Bit &a, const Bit &b) { return a.apos < b.apos; });
-        std::vector<Bit> out;
-        std::vector<char> used(bits.size(), 0);
-        uint32_t span = 1;                        // bank groups reachable: bit set of a subspace of GF(2)^3
-        for (size_t i = 0; i < bits.size() && out.size() < 3; ++i) {
-            const uint32_t g = (bits[i].sm >> 4) & 7u;
-            if ((span >> g) & 1u) continue;       // g is 0 or already in the span
-            uint32_t next = span;
-            for (uint32_t v = 0; v < 8; ++v)
-                if ((span >> v) & 1u) next |= 1u << (v ^ g);
-            span = next;
-            out.push_back(bits[i]);
-            used[i] = 1;
-        }
-        for (size_t i = 0; i < bits.size(); ++i)
-            if (!used[i]) out.push_back(bits[i]);
-        bits = out;
-    };
-    if (!t0 && tpos[0] >= 3) {
-        // qubits 0-2 free: pair bits across the lanes (each instruction 32 consecutive
-        // amplitude pairs of one member), member bits across a thread's copies -- the
-        // order that measured fastest there (10.8 ms per 32-qubit block against 11.4
-        // in address order); the bits are already in that order
-    } else {
-        order(copy);
-        order(store);
-    }
-    RawMap R{};
-    auto fill = [](const std::vector<Bit> &bits, int first, int count, uint64_t *addr, uint32_t *sm, uint32_t *col) {
-        for (int v = 0; v < (1 << count); ++v) {
-            uint64_t a = 0;
-            uint32_t m = 0, c = 0;
-            for (int b = 0; b < count; ++b)
-                if ((v >> b) & 1) {
-                    a |= bits[first + b].addr;
-                    m ^= bits[first + b].sm;
-                    c |= bits[first + b].col;
-                }
-            addr[v] = a;
-            sm[v] = m;
-            col[v] = c;
-        }
-    };
-    fill(copy, 0, 6, R.cthr_addr, R.cthr_sm, R.cthr_col);
-    fill(copy, 6, 6, R.cit_addr, R.cit_sm, R.cit_col);
-    fill(store, 0, 5, R.sl_addr, R.sl_sm, R.sl_col);
-    fill(store, 5, 4, R.sr_addr, R.sr_sm, R.sr_col);
-    (void)n;
-    return R;
-}
-
 template <int P>
 cudaError_t run_tc(const LaunchCtx &L, float2 *sv, const TcGeom &G, const uint4 *d_a, int *d_err) {
     auto kern = k_tc6<P>;
@@ -1194,7 +929,7 @@ cudaError_t launch_tc6(const LaunchCtx &L, void *sv, int n, const int *tpos, con
         // loop's extra instructions per copy cost the copy warps about 13 % there).
         const bool t0 = tpos[0] == 0;
         const bool mapped = !t0 && tpos[0] <= 2 && tpos[1] < 6;
-        const RawMap R = t0 || mapped ? build_raw_map(n, tpos, t0) : RawMap{};
+        const RawMap R = t0 || mapped ? build_raw_map(tpos, tpos, t0, 6) : RawMap{};
         const bool tf = prec == SV_PREC_TF32;
         if (t0) return tf ? run_tc_raw<TF32, RAW_T0>(L, s, G, R, a, d_err, 0) : run_tc_raw<BF16, RAW_T0>(L, s, G, R, a, d_err, 0);
         if (mapped)

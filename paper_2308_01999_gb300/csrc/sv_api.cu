@@ -170,6 +170,8 @@ sv_status_t apply_gate(sv_ctx *h, Gate g, sv_precision_t prec) {
         if (!svk::tc6_supported(h->n, t6.data())) return SV_ERR_NOT_SUPPORTED;
         return cuda_status(svk::launch_tc6(L, h->sv, h->n, t6.data(), m6.data(), prec, h->d_mat, h->d_err));
     }
+    if (h->dt == SV_C64 && k >= 5 && g.c.empty() && svk::tc_x3_ok(h->n, k, flat))
+        return cuda_status(svk::launch_tc_x3(L, h->sv, h->n, g.t.data(), k, flat, h->d_mat, h->d_err));
     return cuda_status(svk::launch_dense(L, h->dt, h->sv, h->n, G, g.t.data(), k, flat, h->d_mat));
 }
 

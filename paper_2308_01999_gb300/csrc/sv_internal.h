@@ -91,6 +91,11 @@ cudaError_t launch_set_basis(const LaunchCtx &L, sv_dtype_t dt, void *sv, int n,
 cudaError_t launch_tc6(const LaunchCtx &L, void *sv, int n, const int *tpos, const double *mat,
                        sv_precision_t prec, void *d_a, int *d_err);
 bool tc6_supported(int n, const int *tpos);
+// Dense 5- or 6-target gate (no controls, targets ascending) at FP32's accuracy on the
+// tensor cores (k_tc_x3.cu), where tc_x3_ok; d_a: workspace of at least 64 KiB.
+bool tc_x3_ok(int n, int k, const double *mat);
+cudaError_t launch_tc_x3(const LaunchCtx &L, void *sv, int n, const int *tpos, int k, const double *mat, void *d_a,
+                         int *d_err);
 // Bounded-wait diagnostic: a wait that nothing completes, limited to `cycles` clocks.
 cudaError_t launch_wait_probe(const LaunchCtx &L, int *d_err, long long cycles);
 
