@@ -429,13 +429,18 @@ template <bool T0 = false>
 __device__ __forceinline__ void split_atom(uint32_t atom, int lane) {
     const int r = lane >> 2, u = lane & 3;          // row, physical 32-byte unit
     const int lu = u ^ (r & 3);                     // logical unit: floats 8 lu .. 8 lu + 7
-    float x[8];
+    // odd rows read their second chunk first: eight lanes (two rows) then cover all
+    // banks (in one order, every load took two wavefronts)
+    float x[8], y[8];
+    const uint32_t src = atom + (uint32_t)(r * 128 + u * 32), odd = (uint32_t)(r & 1) << 4;
     asm volatile("ld.shared.v4.f32 {%0,%1,%2,%3}, [%4];"
-                 : "=f"(x[0]), "=f"(x[1]), "=f"(x[2]), "=f"(x[3])
-                 : "r"(atom + (uint32_t)(r * 128 + u * 32)));
+                 : "=f"(y[0]), "=f"(y[1]), "=f"(y[2]), "=f"(y[3])
+                 : "r"(src + odd));
     asm volatile("ld.shared.v4.f32 {%0,%1,%2,%3}, [%4];"
-                 : "=f"(x[4]), "=f"(x[5]), "=f"(x[6]), "=f"(x[7])
-                 : "r"(atom + (uint32_t)(r * 128 + u * 32 + 16)));
+                 : "=f"(y[4]), "=f"(y[5]), "=f"(y[6]), "=f"(y[7])
+                 : "r"(src + (odd ^ 16u)));
+#pragma unroll
+    for (int k = 0; k < 8; ++k) x[k] = odd ? y[k ^ 4] : y[k];
     if constexpr (T0) {
         // rows 2m, 2m + 1 landed as member pairs of columns 2p, 2p + 1 (qubit 0 a
         // target): trade 8-byte halves with the lane holding the same columns of
@@ -745,10 +750,9 @@ k_tc6_raw(float2 *__restrict__ sv, const TcGeom G, const RawMap R, const uint4 *
                         const float s1 = __shfl_xor_sync(0xffffffffu, even ? o.w : o.y, 1);
                         o = even ? make_float4(o.x, o.y, s0, s1) : make_float4(s0, s1, o.z, o.w);
                     }
-                    // amplitude pair c of the tile, staged as one 16-byte chunk (conflict free:
-                    // the 16 rows of an instruction fall in four 32-byte bank groups)
+                    // amplitude pair c of the tile, staged as one 16-byte chunk
                     const int c = 32 * hh + 8 * cc + 2 * g + e;
-                    asm volatile("st.shared.v4.f32 [%0], {%1,%2,%3,%4};" ::"r"(sb + mn_chunk(j, c)), "f"(o.x),
+                    asm volatile("st.shared.v4.f32 [%0], {%1,%2,%3,%4};" ::"r"(sb + out_chunk(j, c)), "f"(o.x),
                                  "f"(o.y), "f"(o.z), "f"(o.w)
                                  : "memory");
                 }
@@ -772,7 +776,7 @@ k_tc6_raw(float2 *__restrict__ sv, const TcGeom G, const RawMap R, const uint4 *
                     const int c = IL ? 32 * hh + 16 * (r & 1) + pl : cst;
                     asm volatile("ld.shared.v4.f32 {%0,%1,%2,%3}, [%4];"
                                  : "=f"(o.x), "=f"(o.y), "=f"(o.z), "=f"(o.w)
-                                 : "r"(sb + mn_chunk(l, c)));
+                                 : "r"(sb + out_chunk(l, c)));
                     if constexpr (IL) {
                         if ((uint64_t)(2 * c) < G.n_cols)
                             *reinterpret_cast<float4 *>(sv + (tb | (r & 1 ? pst1 : pst0) | G.off[l])) = o;
@@ -921,16 +925,16 @@ cudaError_t launch_tc6(const LaunchCtx &L, void *sv, int n, const int *tpos, con
         const std::vector<unsigned char> img = build_a_image3(mat, prec);
         cudaError_t e = cudaMemcpyAsync(d_a, img.data(), img.size(), cudaMemcpyHostToDevice, L.stream);
         if (e != cudaSuccess) return e;
-        // The copy and store order by target positions (TF32, 32-qubit state, one block):
-        // qubit 0 a target -> RawMap order (14.2-16.1 ms, against 15.8-16.7 for the
-        // register-staged kernel); lowest target 1 or 2 with a second target below 6
-        // -> RawMap order ((1..6) 13.9 ms, (2..7) 11.7, against 16.8 and 13.3 in IL order);
-        // otherwise the fixed orders (lowest target 3 or more: 10.4-10.8 ms; the table
-        // loop's extra instructions per copy cost the copy warps about 13 % there).
+        // The copy and store order by target positions (28-qubit state, one block, TF32 / split
+        // BF16): qubit 0 a target -> RawMap order (1.01 / 0.96 ms, whatever the others);
+        // lowest target 1 -> RawMap order (0.94 / 0.94 ms, IL order 0.97 / 0.96; (1..6) 0.92);
+        // lowest target 2 -> RawMap order in BF16 (0.770, IL 0.788) and where a second target
+        // is below 6, else IL order (TF32 0.760, RawMap 0.775); lowest target 3 -> IL order
+        // (0.705 / 0.748, RawMap 0.775 / 0.793); 4 or more -> PLAIN (0.699 / 0.736).
         const bool t0 = tpos[0] == 0;
-        const bool mapped = !t0 && tpos[0] <= 2 && tpos[1] < 6;
-        const RawMap R = t0 || mapped ? build_raw_map(tpos, tpos, t0, 6) : RawMap{};
         const bool tf = prec == SV_PREC_TF32;
+        const bool mapped = !t0 && (tpos[0] == 1 || (tpos[0] == 2 && (tpos[1] < 6 || !tf)));
+        const RawMap R = t0 || mapped ? build_raw_map(tpos, tpos, t0, 6, 16) : RawMap{};
         if (t0) return tf ? run_tc_raw<TF32, RAW_T0>(L, s, G, R, a, d_err, 0) : run_tc_raw<BF16, RAW_T0>(L, s, G, R, a, d_err, 0);
         if (mapped)
             return tf ? run_tc_raw<TF32, RAW_MAPPED>(L, s, G, R, a, d_err, 0)

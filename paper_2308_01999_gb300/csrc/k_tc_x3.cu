@@ -271,11 +271,6 @@ __device__ __forceinline__ bool convert_half(uint32_t atoms, uint32_t lo_atoms, 
     return true;
 }
 
-// Where the epilogue stages chunk c of row l: mn_chunk with rows 4 .. 7 of an atom in
-// the other 16-byte half of their 32-byte unit, so that the eight rows that eight
-// lanes write fall on all banks
-__device__ __forceinline__ uint32_t out_chunk(int l, int c) { return mn_chunk(l, c) ^ (uint32_t)((l & 4) << 2); }
-
 // Copy and store orders as in k_tc.cu: PLAIN (qubit 0 free, lowest target 4 or
 // more), MAPPED (the table order, qubit 0 free), T0 (qubit 0 a target).
 enum Mode { PLAIN = 0, MAPPED = 1, T0M = 2 };

@@ -130,6 +130,11 @@ __device__ __forceinline__ uint32_t mn_chunk(int l, int c) {
                       ((c & 1) << 4));
 }
 
+// Where the epilogue stages chunk c of row l: mn_chunk with rows 4 .. 7 of an atom in
+// the other 16-byte half of their 32-byte unit, so that the eight rows that eight
+// lanes write fall on all banks
+__device__ __forceinline__ uint32_t out_chunk(int l, int c) { return mn_chunk(l, c) ^ (uint32_t)((l & 4) << 2); }
+
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void *src, uint32_t src_bytes) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(src_bytes) : "memory");
 }
