@@ -403,10 +403,7 @@ constexpr int kFxtThreads = 256;
 template <int K> struct FxtCfg {
     static constexpr int D = 1 << K, ND = K <= 4 ? 7 : 8, B = K <= 4 ? 9 : 8;
     static constexpr int P = K <= 4 ? 61 : 62;
-#ifndef FXB
-#define FXB 2
-#endif
-    static constexpr int blocks = K == 3 ? 3 : K == 4 ? FXB : 1;
+    static constexpr int blocks = K == 3 ? 3 : K == 4 ? 2 : 1;   // resident per SM
     static constexpr int TM = D / 8;             // 16-row tiles of A, and 16-deep steps
     static constexpr size_t smem = sizeof(uint4) * 32 * TM * TM * ND;
 };

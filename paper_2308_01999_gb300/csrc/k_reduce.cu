@@ -413,7 +413,7 @@ cudaError_t sample_t(const LaunchCtx &L, const void *sv, int n, const double *d_
 // a thread (the pair of a complex64 unit, the loads, the iterations) have a
 // partial sum each, lane and warp bits select whole thread totals, and block
 // bits are left to k_zall_finish, which takes one block per qubit. FP32 for
-// complex64 over at most 8 iterations of 16 amplitudes (a tree over the 16),
+// complex64 over at most 4 iterations of 16 amplitudes (a tree over the 16),
 // FP64 beyond; fixed order.
 //
 // What bounds it: HBM; 128 bytes per thread are in flight (27 qubits, complex64:
@@ -421,8 +421,9 @@ cudaError_t sample_t(const LaunchCtx &L, const void *sv, int n, const double *d_
 // block).
 // ---------------------------------------------------------------------------
 constexpr int kZMax = 40;
-constexpr int kZOuter = 20;   // most iteration bits beyond the first three
-constexpr int kZFew = 5;      // the same for states whose blocks take at most 2^8 iterations
+constexpr int kZIn = 2;       // iterations summed in the state's precision: 2^kZIn
+constexpr int kZOuter = 20;   // most iteration bits beyond those
+constexpr int kZFew = 6;      // the same for states whose blocks take at most 2^8 iterations
 
 template <typename R, int MO>
 __global__ void __launch_bounds__(kThreads)
@@ -431,14 +432,14 @@ k_zall(const typename CT<R>::T *__restrict__ sv, uint64_t n_units, int mj, doubl
     constexpr int V = CT<R>::V, vb = V == 2 ? 1 : 0;
     const int t = threadIdx.x;
     const uint64_t u0 = ((uint64_t)blockIdx.x << (11 + mj)) + t;
-    const int inner = mj < 3 ? 1 << mj : 8, mo = mj < 3 ? 0 : mj - 3;
-    double dT = 0.0, dE = 0.0, dL[3] = {0.0, 0.0, 0.0}, dI[3] = {0.0, 0.0, 0.0}, dO[MO > 0 ? MO : 1];
+    const int inner = mj < kZIn ? 1 << mj : 1 << kZIn, mo = mj < kZIn ? 0 : mj - kZIn;
+    double dT = 0.0, dE = 0.0, dL[3] = {0.0, 0.0, 0.0}, dI[kZIn] = {0.0}, dO[MO > 0 ? MO : 1];
 #pragma unroll
     for (int q = 0; q < MO; ++q) dO[q] = 0.0;
     for (uint32_t j = 0; j < (1u << mo); ++j) {
-        R fT = R(0), fE = R(0), fL[3] = {R(0), R(0), R(0)}, fI[3] = {R(0), R(0), R(0)};
+        R fT = R(0), fE = R(0), fL[3] = {R(0), R(0), R(0)}, fI[kZIn] = {R(0)};
         for (int i = 0; i < inner; ++i) {
-            const uint64_t u = u0 + ((uint64_t)(j * 8 + i) << 11);
+            const uint64_t u = u0 + ((uint64_t)((j << kZIn) + i) << 11);
             C a[8][V];
 #pragma unroll
             for (int k = 0; k < 8; ++k) {
@@ -466,16 +467,15 @@ k_zall(const typename CT<R>::T *__restrict__ sv, uint64_t n_units, int mj, doubl
             fL[1] += p23 + p67;
             fL[2] += hi;
 #pragma unroll
-            for (int q = 0; q < 3; ++q)
+            for (int q = 0; q < kZIn; ++q)
                 if ((i >> q) & 1) fI[q] += tot;
         }
         dT += (double)fT;
         dE += (double)fE;
 #pragma unroll
-        for (int q = 0; q < 3; ++q) {
-            dL[q] += (double)fL[q];
-            dI[q] += (double)fI[q];
-        }
+        for (int q = 0; q < 3; ++q) dL[q] += (double)fL[q];
+#pragma unroll
+        for (int q = 0; q < kZIn; ++q) dI[q] += (double)fI[q];
 #pragma unroll
         for (int q = 0; q < MO; ++q)
             if (q < mo && ((j >> q) & 1u)) dO[q] += (double)fT;
@@ -483,7 +483,7 @@ k_zall(const typename CT<R>::T *__restrict__ sv, uint64_t n_units, int mj, doubl
     // block sums in a fixed order: value 0 is the total, value 1 + q the sum over bit q of
     // the block's amplitude index; each warp reduces with shuffles, then thread v adds
     // the warps' results in warp order
-    constexpr int kV = 1 + vb + 5 + 3 + 3 + 3 + MO;
+    constexpr int kV = 1 + vb + 5 + 3 + 3 + kZIn + MO;
     __shared__ double wred[kThreads / 32][kV];
     const int lane = t & 31, warp = t >> 5;
     const int nv = 1 + vb + 11 + mj;
@@ -514,11 +514,11 @@ k_zall(const typename CT<R>::T *__restrict__ sv, uint64_t n_units, int mj, doubl
 #pragma unroll
     for (int q = 0; q < 3; ++q) warp_put(dL[q], 1 + vb + 8 + q);
 #pragma unroll
-    for (int q = 0; q < 3; ++q)
+    for (int q = 0; q < kZIn; ++q)
         if (q < mj) warp_put(dI[q], 1 + vb + 11 + q);
 #pragma unroll
     for (int q = 0; q < MO; ++q)
-        if (q < mo) warp_put(dO[q], 1 + vb + 14 + q);
+        if (q < mo) warp_put(dO[q], 1 + vb + 11 + kZIn + q);
     __syncthreads();
     if (t < nv) {
         double acc = 0.0;
@@ -572,9 +572,9 @@ cudaError_t zall_t(const LaunchCtx &L, const void *sv, int n, double *d_partials
     const int mj = ub > 11 + zb ? ub - 11 - zb : 0;
     const uint64_t n_units = 1ull << ub;
     const uint64_t blocks = ub > 11 ? n_units >> (11 + mj) : 1;
-    if (mj > 3 + kZOuter || blocks * (uint64_t)(1 + vb + 11 + mj) > (uint64_t)maxb * 8) return cudaErrorInvalidValue;
+    if (mj > kZIn + kZOuter || blocks * (uint64_t)(1 + vb + 11 + mj) > (uint64_t)maxb * 8) return cudaErrorInvalidValue;
     // the sums of the outer iteration bits take two registers each
-    auto kern = mj <= 3 + kZFew ? k_zall<R, kZFew> : k_zall<R, kZOuter>;
+    auto kern = mj <= kZIn + kZFew ? k_zall<R, kZFew> : k_zall<R, kZOuter>;
     kern<<<(unsigned)blocks, kThreads, 0, L.stream>>>(reinterpret_cast<const C *>(sv), n_units, mj, d_partials);
     ++*L.launches;
     cudaError_t e = cudaGetLastError();
