@@ -546,6 +546,130 @@ __device__ __forceinline__ double pauli_terms(const float2 *tile, const float2 *
     return acc;
 }
 
+// R strings with independent X/Y masks in one pass over chunk c of nch: a thread
+// reads the 2^R amplitudes i ^ span(x_0 .. x_{R-1}) of a coset once and has every
+// string's 2^(R-1) pairs in registers (string k pairs members that differ in bit
+// k). The pairs' signs are one sign per other mask times the coset's own; a
+// string's sum over a coset is a tree of FP32 terms, accumulated per thread in
+// FP32 with compensation (an FP64 addition per eight amplitudes and string took
+// as long as reading them), FP64 across threads. The totals of the block come
+// back in thread 0's tot. (600 circuits of 10 to 20 qubits, 8 strings each: the
+// launch takes BNOTE.)
+template <int R, bool CG>
+__device__ __noinline__ void pauli_group(const float2 *tile, const float2 *sv, bool in_tile, const BStr *strs, int n,
+                                         uint32_t c, uint32_t nch, double *red, double (&tot)[R]) {
+    constexpr int N = 1 << R;
+    uint32_t x[R], z[R], off[N], piv[R];
+    bool im[R];
+#pragma unroll
+    for (int k = 0; k < R; ++k) {
+        x[k] = (uint32_t)strs[k].x;
+        z[k] = (uint32_t)strs[k].z;
+        im[k] = strs[k].use_im != 0;
+    }
+    off[0] = 0;
+#pragma unroll
+    for (int j = 1; j < N; ++j) {
+        const int b = 31 - __clz(j);
+        off[j] = off[j ^ (1 << b)] ^ x[b];
+    }
+    // a reduced basis of the masks gives one bit position per vector that is zero in one
+    // member of every coset; high ones keep a warp's reads contiguous
+    uint32_t v[R];
+#pragma unroll
+    for (int k = 0; k < R; ++k) {
+        v[k] = x[k];
+#pragma unroll
+        for (int l = 0; l < k; ++l)
+            if ((v[k] >> piv[l]) & 1u) v[k] ^= v[l];
+        piv[k] = 31 - __clz(v[k]);
+#pragma unroll
+        for (int l = 0; l < k; ++l)
+            if ((v[l] >> piv[k]) & 1u) v[l] ^= v[k];
+    }
+    uint32_t pmask = 0;
+#pragma unroll
+    for (int k = 0; k < R; ++k) pmask |= 1u << piv[k];
+    float sg[R][R];                                     // sign of mask b in string k's pairs
+#pragma unroll
+    for (int k = 0; k < R; ++k)
+#pragma unroll
+        for (int b = 0; b < R; ++b) sg[k][b] = (__popc(x[b] & z[k]) & 1) ? -1.f : 1.f;
+    float acc[R], cmp[R];
+#pragma unroll
+    for (int k = 0; k < R; ++k) acc[k] = cmp[k] = 0.f;
+    const uint32_t per = (1u << (n - R)) / nch;
+    for (uint32_t g = c * per + threadIdx.x; g < (c + 1) * per; g += kT) {
+        uint32_t i = g;
+        uint32_t pm = pmask;
+#pragma unroll
+        for (int k = 0; k < R; ++k) {                   // a zero at each pivot, lowest first
+            const uint32_t low = (pm & (0u - pm)) - 1u;
+            i = ((i & ~low) << 1) | (i & low);
+            pm &= pm - 1u;
+        }
+        float2 a[N];
+#pragma unroll
+        for (int j = 0; j < N; ++j) {
+            const uint32_t q = i ^ off[j];
+            if constexpr (CG) a[j] = __ldcg(sv + q);
+            else a[j] = in_tile ? tile[sw(q)] : sv[q];
+        }
+#pragma unroll
+        for (int k = 0; k < R; ++k) {
+            float t[N / 2];
+#pragma unroll
+            for (int p = 0; p < N / 2; ++p) {           // p: the member's other bits
+                const int j = ((p >> k) << (k + 1)) | (p & ((1 << k) - 1)), l = j | (1 << k);
+                t[p] = im[k] ? __fmaf_rn(a[j].y, a[l].x, -(a[j].x * a[l].y)) : __fmaf_rn(a[j].x, a[l].x, a[j].y * a[l].y);
+            }
+            int w = N / 2;
+#pragma unroll
+            for (int b = 0; b < R; ++b) {               // fold the other masks' bits, lowest first
+                if (b == k) continue;
+                w >>= 1;
+#pragma unroll
+                for (int p = 0; p < N / 4; ++p)
+                    if (p < w) t[p] = __fmaf_rn(t[2 * p + 1], sg[k][b], t[2 * p]);
+            }
+            const float y = (__popc(i & z[k]) & 1) ? -t[0] : t[0];
+            const float u = acc[k] + y;
+            cmp[k] += fabsf(acc[k]) >= fabsf(y) ? (acc[k] - u) + y : (y - u) + acc[k];
+            acc[k] = u;
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < R; ++k) tot[k] = block_sum(2.0 * ((double)acc[k] + (double)cmp[k]), red);
+}
+
+// how many of the strings from s on share a pass: 3 or 2 with independent masks, else 1
+__device__ __forceinline__ int group_of(const BStr *strs, int left, int n) {
+    if (n < 4 || left < 2) return 1;
+    const uint64_t a = strs[0].x, b = strs[1].x;
+    if (a == 0 || b == 0 || a == b) return 1;
+    if (left < 3) return 2;
+    const uint64_t c = strs[2].x;
+    return c != 0 && c != a && c != b && c != (a ^ b) ? 3 : 2;
+}
+
+// chunk c of nch of the strings that share the next pass (cnt of them); totals in thread 0's tot
+template <bool CG>
+__device__ __forceinline__ void chunk_sums(const float2 *tile, const float2 *sv, bool in_tile, const BStr *strs, int cnt, int n,
+                                           uint32_t c, uint32_t nch, double *red, double (&tot)[3]) {
+    if (cnt == 3) {
+        pauli_group<3, CG>(tile, sv, in_tile, strs, n, c, nch, red, tot);
+    } else if (cnt == 2) {
+        double two[2];
+        pauli_group<2, CG>(tile, sv, in_tile, strs, n, c, nch, red, two);
+        tot[0] = two[0];
+        tot[1] = two[1];
+    } else {
+        const BStr Ps = strs[0];
+        const uint32_t per = (Ps.x ? (1u << n) / 2 : (1u << n)) / nch;
+        tot[0] = block_sum(pauli_terms<CG>(tile, sv, in_tile, Ps, c * per, (c + 1) * per), red);
+    }
+}
+
 // Thread 0 waits (bounded) until `need` tile tasks of the item have finished;
 // then every thread may read what they wrote. False when the wait gave up or
 // another CTA had already given up.
@@ -637,12 +761,13 @@ __device__ __noinline__ void task_expect(BSmem &sh, float2 *states, const BProg 
     const float2 *sv = states + it.state_off;
     const int n = it.n;
     const uint32_t c = tk.a, nch = (uint32_t)it.n_chunks;
-    for (int s = 0; s < it.n_str; ++s) {
-        const BStr Ps = P.strs[it.str_begin + s];
-        const uint32_t npairs = Ps.x ? (1u << n) / 2 : (1u << n);
-        const uint32_t per = npairs / nch;
-        const double tot = block_sum(pauli_terms<true>(nullptr, sv, false, Ps, c * per, (c + 1) * per), sh.red);
-        if (threadIdx.x == 0) P.parts[it.part_begin + c * it.n_str + s] = tot;
+    for (int s = 0, cnt; s < it.n_str; s += cnt) {
+        const BStr *strs = P.strs + it.str_begin + s;
+        cnt = group_of(strs, it.n_str - s, n);
+        double tot[3];
+        chunk_sums<true>(nullptr, sv, false, strs, cnt, n, c, nch, sh.red, tot);
+        if (threadIdx.x == 0)
+            for (int k = 0; k < cnt; ++k) P.parts[it.part_begin + c * it.n_str + s + k] = tot[k];
     }
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -712,15 +837,17 @@ __device__ __forceinline__ void run_state(float2 *tile, float2 *smat, BSmem &sh,
         }
     }
     const uint32_t nch = n == T ? 1u : (uint32_t)it.n_chunks;
-    for (int s = 0; s < it.n_str; ++s) {
-        const BStr Ps = P.strs[it.str_begin + s];
-        const uint32_t npairs = Ps.x ? (1u << n) / 2 : (1u << n);
-        const uint32_t per = npairs / nch;
-        double t = 0.0;
+    for (int s = 0, cnt; s < it.n_str; s += cnt) {
+        const BStr *strs = P.strs + it.str_begin + s;
+        cnt = group_of(strs, it.n_str - s, n);
+        double t[3] = {0.0, 0.0, 0.0};
         for (uint32_t c = 0; c < nch; ++c) {
-            t += block_sum(pauli_terms<false>(tile, sv, n == T, Ps, c * per, (c + 1) * per), sh.red);
+            double tot[3];
+            chunk_sums<false>(tile, sv, n == T, strs, cnt, n, c, nch, sh.red, tot);
+            for (int k = 0; k < cnt; ++k) t[k] += tot[k];
         }
-        if (threadIdx.x == 0) P.out[it.out_begin + s] = (double)Ps.sign * t;
+        if (threadIdx.x == 0)
+            for (int k = 0; k < cnt; ++k) P.out[it.out_begin + s + k] = (double)strs[k].sign * t[k];
     }
 }
 
