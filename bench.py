@@ -68,8 +68,10 @@ def gate_bytes(g):
 
 
 def reduction_passes(paulis):
-    """Passes over the state: <Z_q> (x = 0, 8 strings per pass), the Pauli strings
-    grouped by their X/Y mask (8 per pass), and one parity pass."""
+    """Passes the step's bytes are counted with: <Z_q> (x = 0, 8 strings per pass),
+    the Pauli strings grouped by their X/Y mask (8 per pass), and one parity pass.
+    The kernels make fewer (all <Z_q> in one, several masks in one); the count is
+    kept so that values stay comparable: it is 0.5 % of the step's bytes."""
     zpasses = (N_QUBITS + 7) // 8
     xs = {}
     for p in paulis:

@@ -19,7 +19,7 @@
 // The pipeline is k_tc6_raw's (k_tc.cu): the 64 members of a group are the
 // contraction, the state tile is the MN-major B operand, its rows are re and im
 // of 64 columns; 2 copy warps (cp.async into the stage, arriving on `landed`),
-// 4 convert warps (digits in place: a 1 KiB atom of 8 members x 32 floats
+// 8 convert warps (digits in place: a 1 KiB atom of 8 members x 32 floats
 // becomes its hi and mid atoms, lo atoms go to 16 KiB of their own), one MMA
 // thread, 8 epilogue warps that add the accumulators, combine the Re and Im
 // rows, stage the result where the tile came from and store it. Tiles are 64
