@@ -81,7 +81,8 @@ __device__ __forceinline__ uint64_t mant64(int hi, int lo) {
 // The x0 m0 products (below 2^-59 of the full scale, random sign) are dropped.
 //
 // What bounds it: HBM, with the integer pipes close behind (about 80 ALU and
-// 24 / 48 multiply-add instructions per amplitude).
+// 24 / 48 multiply-add instructions per amplitude). 26 qubits (HBM 0.316 ms):
+// 0.32 to 0.34 ms for k = 1 (FP64 1.02), 0.44 to 0.46 for k = 2 (FP64 2.03).
 // ---------------------------------------------------------------------------
 template <int K> struct Fx2 {
     static constexpr int P = 61 - K, PM = 61 - K;
@@ -184,7 +185,9 @@ k_dense_fx2(double2 *__restrict__ sv, uint64_t n_groups, GroupGeom G, Offs<K> O,
 //
 // What bounds it: the integer multiply-adds (18 per complex product; one
 // thread holds a group of up to 16 amplitudes in limbs, the matrix is
-// broadcast from shared memory, 24 bytes per complex product).
+// broadcast from shared memory, 24 bytes per complex product). 26 qubits: 1.02 ms
+// for k = 2 (FP64 2.03), 2.98 for k = 4 (FP64 8.1; four lanes a group or other
+// occupancies up to 3.46).
 // ---------------------------------------------------------------------------
 constexpr int kL = 28;
 constexpr int kFx3Threads = 128;
@@ -396,7 +399,10 @@ k_dense_fx3(double2 *__restrict__ sv, uint64_t n_groups, GroupGeom G, const __gr
 // store instruction covers 64 contiguous bytes per member.
 //
 // What bounds it: conversions to digits and back (about 110 instructions per
-// amplitude) and the MMAs, close to the time of the 32 bytes an amplitude moves.
+// amplitude; ALU 46 %, FP64 25 % busy at k = 4) and the MMAs (53 %), which the 16 to
+// 24 warps of an SM overlap in part; the 32 bytes an amplitude moves are a third to a
+// half of the time. 26 qubits: 0.75 ms for k = 3, 0.90 for k = 4, 2.0 for k = 5 (FP64
+// 4.06, 8.1, 14.0; three limbs 2.98 at k = 4). Three blocks per SM at k = 4: 1.01.
 // ---------------------------------------------------------------------------
 constexpr int kFxtThreads = 256;
 
@@ -742,6 +748,10 @@ bool try_dense_fx(const LaunchCtx &L, void *sv, int n, const GroupGeom &G, const
     if (k > 5) return false;
     const MatRange r = range_of(mat, 1 << (2 * k));
     if (!r.finite || r.em < -100 || r.em > 100) return false;
+    // The lines are where each layout's error bound ends (above), not where the times
+    // cross: the first that may run is the fastest. 26 qubits, ms: two limbs 0.32 / 0.44
+    // (k = 1, 2), digits 0.75 / 0.90 / 2.0 (k = 3, 4, 5), three limbs 1.02 / 2.98 (k = 2,
+    // 4), FP64 1.02 / 2.03 / 4.06 / 8.1 / 14.0. k = 6 stays in FP64.
     const uint64_t n_groups = 1ull << (n - G.ns);
     if (k <= 2 && !r.zeros && r.dm <= (k == 1 ? 6 : 5)) {
         e = k == 1 ? run_fx2<1>(L, sv, n_groups, G, tpos, mat, r.em) : run_fx2<2>(L, sv, n_groups, G, tpos, mat, r.em);
