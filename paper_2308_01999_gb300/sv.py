@@ -509,7 +509,12 @@ def pack_gates(gates, square: bool = False):
             rec["targets"][idx, :k] = table([targets[i] for i in members], k)
         if c:
             rec["controls"][idx, :c] = table([controls[i] for i in members], c)
-            rec["control_values"][idx, :c] = table([gates[i].control_values or (1,) * c for i in members], c)
+            values = [gates[i].control_values or (1,) * c for i in members]
+            if set(map(len, values)) != {c}:        # more than c: the rest is ignored, as in sv_apply_matrix
+                values = [tuple(v)[:c] for v in values]
+                if min(map(len, values)) < c:
+                    raise IndexError("fewer control values than controls")
+            rec["control_values"][idx, :c] = table(values, c)
     return rec, buf
 
 
