@@ -487,11 +487,11 @@ def pack_gates(gates, square: bool = False):
     groups = {}
     for i, key in enumerate(zip(map(len, targets), map(len, controls))):
         groups.setdefault(key, []).append(i)
+    if any(k > SV_MAX_TARGETS or c > SV_MAX_CONTROLS for k, c in groups):
+        raise IndexError("too many targets or controls")
     buf = np.empty(sum(len(members) << (2 * k) for (k, _), members in groups.items()), dtype=np.complex128)
     at = 0
     for (k, c), members in groups.items():
-        if k > SV_MAX_TARGETS or c > SV_MAX_CONTROLS:
-            raise IndexError("too many targets or controls")
         idx = slice(None) if len(groups) == 1 else np.array(members)
         n, d = len(members), 1 << k
         mats = [matrices[i] for i in members]

@@ -33,3 +33,9 @@ def test_missing_control_values_are_an_error(lengths):
         sv.pack_gates(gates)
     with pytest.raises((IndexError, ValueError)):
         sv.sv_fuse_plan(gates, 4, 2)
+
+
+def test_too_many_targets_is_an_index_error():
+    """Not an attempt to allocate 4^k entries."""
+    with pytest.raises(IndexError):
+        sv.pack_gates([G(tuple(range(24)), X, (), ())])
