@@ -192,6 +192,8 @@ def sv_apply_matrix(h: int, targets, matrix, controls=(), control_values=None, a
     c, cp = _ints(controls)
     if control_values is not None and len(control_values):
         cv, cvp = _ints(control_values)
+        if cv.size < c.size:
+            raise ValueError("fewer control values than controls")
     else:
         cv, cvp = None, None
     m, mp = _cmat(matrix)

@@ -39,3 +39,8 @@ def test_too_many_targets_is_an_index_error():
     """Not an attempt to allocate 4^k entries."""
     with pytest.raises(IndexError):
         sv.pack_gates([G(tuple(range(24)), X, (), ())])
+
+
+def test_missing_control_values_in_the_direct_call():
+    with pytest.raises(ValueError):
+        sv.sv_apply_matrix(0, (0,), X, (1, 2), (1,))
