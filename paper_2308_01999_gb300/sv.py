@@ -402,11 +402,16 @@ class StateVector:
         sv_apply_matrix(self.handle, g.targets, g.matrix, g.controls, g.control_values or None, adjoint)
 
     def apply_circuit(self, gates):
-        gates = list(gates)
-        try:
-            arr, _keep = _gate_array(gates, square=True)
-        except (TypeError, ValueError, IndexError, AttributeError):
-            for g in gates:         # a gate that cannot be packed: the ones before it still apply
+        """A list or tuple of gates in one native call; other iterables gate by gate, each asked for its next
+        gate after the one before has been applied (a generator may look at the state)."""
+        arr = None
+        if isinstance(gates, (list, tuple)) and type(self).apply_gate is StateVector.apply_gate:
+            try:
+                arr, _keep = _gate_array(gates, square=True)
+            except Exception:       # a gate that cannot be packed: the ones before it still apply
+                pass
+        if arr is None:
+            for g in gates:
                 self.apply_gate(g)
             return
         _check(lib().sv_apply_circuit(_VP(self.handle), arr, len(gates)), "sv_apply_circuit")
