@@ -4,42 +4,48 @@
 // On CUDA cores these gates are bound by the FP32 pipe (128 / 256 FMAs per
 // amplitude against 16 bytes moved; k_gate.cu). Here both operands are cut into
 // BF16 digits and the product is the sum of digit products:
-//   state column: x = hi + mid + lo. With X a power of two above the column's
-//     largest value, hi is x rounded to a multiple of X 2^-7, mid the rest rounded
-//     to a multiple of X 2^-15, lo the rest rounded to BF16 (|x - sum| < X 2^-25);
-//   matrix row:   four digits in the same way, below 2^-33 of the row's largest.
+//   state: x = hi + mid + two more. With X a power of two above the largest of the
+//     real (or of the imaginary) parts of the column, hi is x rounded to a multiple
+//     of X 2^-7, mid the rest rounded to a multiple of X 2^-15, and what is left is
+//     rounded to BF16 twice (|x - sum| < X 2^-34). A column is one group of 64
+//     amplitudes; its real and imaginary parts are operand rows of their own, so
+//     neither other groups nor, under a real matrix, the other parts enter the error;
+//   matrix row (real or imaginary parts): four digits in the same way, below 2^-34 of
+//     the row's largest.
 // hi times hi is summed in an accumulator of its own: all its terms are
 // multiples of one unit and the sum stays below 2^20 of them, so it is exact
 // whatever rounding the tensor core's FP32 accumulation does (a truncating sum
 // of the whole product would shrink the norm by a constant per gate). The other
-// products (digits i, j from the top with i + j <= 3) are at most 2^-7 of the
-// first, go into a second accumulator smallest first, and the two are added with
-// one rounding. Measured error per gate: see the rule in tc_x3_ok().
+// products (digits i, j from the top with i + j <= 4: 12 kinds) are at most 2^-7 of
+// the first, go into a second accumulator smallest first, and the two are added
+// with one rounding. Error per gate: see the
+// rule in tc_x3_ok(). Three state digits and nine products (0.98 to 1.00 ms a gate on
+// 28 qubits) kept 25 bits below X: where one amplitude dominates a group the small
+// outputs then had up to 700 u sum |m||x|.
 //
 // The pipeline is k_tc6_raw's (k_tc.cu): the 64 members of a group are the
 // contraction, the state tile is the MN-major B operand, its rows are re and im
 // of 64 columns; 2 copy warps (cp.async into the stage, arriving on `landed`),
 // 8 convert warps (digits in place: a 1 KiB atom of 8 members x 32 floats
-// becomes its hi and mid atoms, lo atoms go to 16 KiB of their own), one MMA
-// thread, 8 epilogue warps that add the accumulators, combine the Re and Im
-// rows, stage the result where the tile came from and store it. Tiles are 64
-// columns (32 KiB): four stages of 48 KiB. The matrix is in TMEM, beside the
-// accumulators of one tile, because the shared-memory port is what the roles share.
+// becomes its hi and mid atoms, the other two go to one of two 32 KiB buffers that
+// the products give back), one MMA thread, 8 epilogue warps that add the
+// accumulators, combine the Re and Im rows, stage the result where the tile came
+// from and store it. Tiles are 64 columns (32 KiB), in four stages. The matrix is in
+// TMEM, beside the accumulators, because the shared-memory port is what the roles
+// share. The twelve small kinds of two tiles have an accumulator each, so the next
+// tile's can run while the epilogue reads this one (with one: 1.46 ms a gate, 1.13 so).
 //
 // A 5-target gate takes one more qubit as the top member bit with an identity:
 // the block-diagonal product keeps its halves apart, and each half of a column
 // has its own X.
 //
-// What bounds it: the roles' latencies in turn. Per tile of 64 columns the tensor pipe
-// is busy 2400 clocks (36 MMAs; it waits while the epilogue reads the one set of
-// accumulators), HBM needs 3000, and the shared-memory port is about 65 % busy at
-// 4100. 28 qubits, one gate: 1.00 ms for k = 6 (k_dense6 3.21) and 0.98 ms for k = 5
-// (k_dense5 1.40); 1.20 and 1.15 ms with qubit 0 a target (3.3 and 1.37). On the way
-// (k = 6): digits by 4 convert warps 1.31 ms; by 8 that hold their atoms in registers,
-// without bank conflicts, 1.21; the matrix in TMEM instead of shared memory 1.15; no
-// ragged tiles 1.00. Three half-tile accumulators in turn were slower (1.33: an N = 64
-// MMA takes as long as an N = 128 one), as was reading the whole accumulator ahead
-// of the combination (1.15 to 1.65, spills).
+// What bounds it: the tensor pipe, busy 3430 clocks per tile of 64 columns (52 MMAs),
+// and the conversion that feeds it, of about 5200 in all; HBM needs 3000. 28 qubits,
+// one gate: 1.13 to 1.16 ms for k = 6 (k_dense6 3.30) and 1.08 to 1.10 ms for k = 5
+// (k_dense5 1.40); 1.17 to 1.21 and 1.13 to 1.15 ms with qubit 0 a target (3.24 and
+// 1.36). N = 64 MMAs (half-tile accumulators) take as long as N = 128 ones; digits by
+// 4 convert warps instead of 8 that hold their atoms in registers, the matrix in shared
+// memory and ragged tiles were each slower.
 #include <cuda_bf16.h>
 
 #include <cmath>
@@ -55,28 +61,28 @@ constexpr int kStages = 4;
 constexpr int kDigA = 4;
 constexpr int kADigit = 128 * 64 * 2;         // one digit of A: 128 rows x 64 BF16
 constexpr int kA = kDigA * kADigit;
-constexpr int kRaw = 64 * 2 * kNT * 4;        // a tile: 64 members x 128 floats
-constexpr int kLo = 64 * 2 * kNT * 2;         // its lo digits
-constexpr int kStage = kRaw + kLo;
+constexpr int kRaw = 64 * 2 * kNT * 4;        // a tile: 64 members x 128 floats, then its first two digits
+constexpr int kLow = kRaw;                    // its last two digits, laid out alike
+constexpr int kLows = 2;                      // buffers of those, held from the conversion to the end of the products
 constexpr int kCopyWarps = 2, kConvWarps = 8, kEpiWarps = 8;
 constexpr int kProdWarps = kCopyWarps + kConvWarps;
 constexpr int kMmaWarp = kProdWarps + kEpiWarps;
 constexpr int kThreads = (kMmaWarp + 1) * 32;
-constexpr int kAccCols = 2 * 2 * kNT;         // hi hi and the rest, 128 columns each
+constexpr int kAccCols = 3 * 2 * kNT;         // hi hi, and the rest of two tiles in turn, 128 columns each
 constexpr int kACols = kDigA * 32;            // A in TMEM: row m in lane m, two BF16 per column
-constexpr int kTmemCols = 512;                // A, then the accumulators of one tile
+constexpr int kTmemCols = 512;                // A, then the accumulators
 static_assert(kACols + kAccCols <= kTmemCols, "TMEM");
 
 struct Ctl {
-    unsigned long long landed[kStages], full[kStages], empty[kStages], acc_full, acc_empty, xch[4], done;
+    unsigned long long landed[kStages], full[kStages], empty[kStages], low_free[kLows], acc_full, acc_empty, xch[4], done;
     // non-finite columns of a stage: half of the members, column block; bit c: column c of the block's 16
     unsigned bad[kStages][2][4];
-    uint32_t share[2][4][2][8];               // maxima of a column block's halves, two tiles in turn
+    uint32_t share[2][4][2][16];              // maxima of a column block's halves, two tiles in turn
     unsigned tmem_base;
     int abort;
 };
-constexpr int kGuard = 2048;                  // unused bytes after the last stage
-constexpr int kSmem = kStages * kStage + kGuard + (int)sizeof(Ctl);
+constexpr int kGuard = 2048;                  // unused bytes after the last buffer
+constexpr int kSmem = kStages * kRaw + kLows * kLow + kGuard + (int)sizeof(Ctl);
 static_assert(kSmem <= 227 * 1024, "dynamic shared memory of the kernel exceeds the per-block limit");
 
 // MN-major operand descriptor of BF16 atoms (8 members x 32 columns, 64-byte
@@ -174,64 +180,67 @@ __device__ __forceinline__ void load8(uint32_t addr, int r, float (&x)[8]) {
 // Half of a column block (32 floats x 32 members, 4 atoms 1 KiB apart) of a landed
 // stage into its digits, by one warp, the atoms held in registers. A lane's chunks
 // are columns 4 lu .. 4 lu + 3 of row r; lanes with the same lu (lane ^ 5, ^ 10,
-// ^ 16) hold the other rows. The scale is common to a chunk's two columns and to
-// all members (the two warps of a block trade their maxima through `share` and
-// the block's barrier), or to the members of one half (halves).
+// ^ 16) hold the other rows. The real and the imaginary parts of every column have
+// a scale each, common to all members (the two warps of a block trade their maxima
+// through `share` and the block's barrier), or to the members of one half (halves).
 template <bool T0>
-__device__ __forceinline__ bool convert_half(uint32_t atoms, uint32_t lo_atoms, int lane, int half, int halves,
-                                             volatile uint32_t (*share)[8], uint32_t xch, uint32_t parity, unsigned *bad,
+__device__ __forceinline__ bool convert_half(uint32_t atoms, uint32_t low_atoms, int lane, int half, int halves,
+                                             volatile uint32_t (*share)[16], uint32_t xch, uint32_t parity, unsigned *bad,
                                              volatile int *abort_flag, int *d_err) {
     const int r = lane >> 2, u = lane & 3, lu = u ^ (r & 3);
     const uint32_t src = (uint32_t)(r * 128 + u * 32), dst = (uint32_t)(r * 64 + ((lu ^ ((r >> 1) & 3)) << 4));
     float x[4][8];
-    uint32_t top[2] = {0, 0};                            // per chunk: largest magnitude as bits
+    uint32_t top[4] = {0, 0, 0, 0};                      // per column: the upper 16 bits of its largest real and imaginary part
 #pragma unroll
     for (int g = 0; g < 4; ++g) {
         load8<T0>(atoms + (uint32_t)(g * 1024) + src, r, x[g]);
 #pragma unroll
-        for (int k = 0; k < 8; ++k) top[k >> 2] = max(top[k >> 2], __float_as_uint(x[g][k]) & 0x7fffffffu);
+        for (int c = 0; c < 4; ++c)
+            top[c] = __vmaxu2(top[c], __byte_perm(__float_as_uint(x[g][2 * c]), __float_as_uint(x[g][2 * c + 1]), 0x7632) &
+                                          0x7fff7fffu);
     }
 #pragma unroll
-    for (int c = 0; c < 2; ++c) {
-        top[c] = max(top[c], __shfl_xor_sync(0xffffffffu, top[c], 5));
-        top[c] = max(top[c], __shfl_xor_sync(0xffffffffu, top[c], 10));
-        top[c] = max(top[c], __shfl_xor_sync(0xffffffffu, top[c], 16));
+    for (int c = 0; c < 4; ++c) {
+        top[c] = __vmaxu2(top[c], __shfl_xor_sync(0xffffffffu, top[c], 5));
+        top[c] = __vmaxu2(top[c], __shfl_xor_sync(0xffffffffu, top[c], 10));
+        top[c] = __vmaxu2(top[c], __shfl_xor_sync(0xffffffffu, top[c], 16));
     }
     if (!halves) {
         if (lane < 4) {                                  // row 0: lu = lane
-            share[half][2 * lane] = top[0];
-            share[half][2 * lane + 1] = top[1];
+#pragma unroll
+            for (int c = 0; c < 4; ++c) share[half][4 * lane + c] = top[c];
         }
         mbar_arrive(xch);
         if (!mbar_wait(xch, parity, abort_flag, d_err)) return false;
-        top[0] = max(top[0], share[half ^ 1][2 * lu]);
-        top[1] = max(top[1], share[half ^ 1][2 * lu + 1]);
+#pragma unroll
+        for (int c = 0; c < 4; ++c) top[c] = __vmaxu2(top[c], share[half ^ 1][4 * lu + c]);
     }
-    float c1[2], c2[2];
+    float c1[8];                                         // unit X 2^-7; X 2^-15 is 2^-8 of it
     bool in = true;
 #pragma unroll
-    for (int c = 0; c < 2; ++c) {
+    for (int k = 0; k < 8; ++k) {
         // X = 2^(e - 126); adding and taking away 1.5 2^23 units rounds to a multiple of a unit
-        const uint32_t e = top[c] >> 23;
-        const bool ok = e >= 40 && e <= 230;
-        in = in && (ok || top[c] == 0);
-        c1[c] = ok ? __uint_as_float(((e + 17u) << 23) | 0x400000u) : 0.f;            // unit X 2^-7
-        c2[c] = ok ? __uint_as_float(((e + 9u) << 23) | 0x400000u) : 0.f;             // unit X 2^-15
+        const uint32_t t = (k & 1) ? top[k >> 1] >> 16 : top[k >> 1] & 0xffffu, e = t >> 7;
+        const bool ok = (e >= 40 && e <= 230) || t == 0;
+        in = in && ok;
+        c1[k] = ok ? __uint_as_float((((t == 0 ? 40u : e) + 17u) << 23) | 0x400000u) : 0.f;
     }
+    auto second = [](float a) { return __uint_as_float(__float_as_uint(a) - (8u << 23)); };
     if (lane == 0) *bad = 0;
     const bool all_in = __all_sync(0xffffffffu, in);
     unsigned nf = 0;
 #pragma unroll
     for (int g = 0; g < 4; ++g) {
-        float hi[8], mid[8], lo[8];
-        uint32_t dh[4], dm[4], dl[4];
+        float hi[8], mid[8], rest[8];
+        uint32_t d[4][4];
         if (all_in) {
 #pragma unroll
             for (int k = 0; k < 8; ++k) {
-                hi[k] = __fsub_rn(__fadd_rn(x[g][k], c1[k >> 2]), c1[k >> 2]);
-                const float rest = __fsub_rn(x[g][k], hi[k]);
-                mid[k] = __fsub_rn(__fadd_rn(rest, c2[k >> 2]), c2[k >> 2]);
-                lo[k] = __fsub_rn(rest, mid[k]);
+                hi[k] = __fsub_rn(__fadd_rn(x[g][k], c1[k]), c1[k]);
+                rest[k] = __fsub_rn(x[g][k], hi[k]);
+                const float c2 = second(c1[k]);
+                mid[k] = __fsub_rn(__fadd_rn(rest[k], c2), c2);
+                rest[k] = __fsub_rn(rest[k], mid[k]);
             }
         } else {
             // columns beyond the range of the scales: digits by rounding to BF16 (their
@@ -244,28 +253,29 @@ __device__ __forceinline__ bool convert_half(uint32_t atoms, uint32_t lo_atoms, 
                     nf |= 1u << (4 * lu + (k >> 1));
                     v = 0.f;
                 }
-                const float a = c1[k >> 2], b = c2[k >> 2];
+                const float a = c1[k], b = second(a);
                 hi[k] = a != 0.f ? __fsub_rn(__fadd_rn(v, a), a) : bf16_part(v);
-                const float rest = __fsub_rn(v, hi[k]);
-                mid[k] = b != 0.f ? __fsub_rn(__fadd_rn(rest, b), b) : bf16_part(rest);
-                lo[k] = __fsub_rn(rest, mid[k]);
+                rest[k] = __fsub_rn(v, hi[k]);
+                mid[k] = a != 0.f ? __fsub_rn(__fadd_rn(rest[k], b), b) : bf16_part(rest[k]);
+                rest[k] = __fsub_rn(rest[k], mid[k]);
             }
         }
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
             // hi and mid are BF16 numbers: their upper halves
-            dh[k] = __byte_perm(__float_as_uint(hi[2 * k]), __float_as_uint(hi[2 * k + 1]), 0x7632);
-            dm[k] = __byte_perm(__float_as_uint(mid[2 * k]), __float_as_uint(mid[2 * k + 1]), 0x7632);
-            dl[k] = bf16x2(lo[2 * k], lo[2 * k + 1]);
+            d[0][k] = __byte_perm(__float_as_uint(hi[2 * k]), __float_as_uint(hi[2 * k + 1]), 0x7632);
+            d[1][k] = __byte_perm(__float_as_uint(mid[2 * k]), __float_as_uint(mid[2 * k + 1]), 0x7632);
+            d[2][k] = bf16x2(rest[2 * k], rest[2 * k + 1]);
+            d[3][k] = bf16x2(__fsub_rn(rest[2 * k], __uint_as_float(d[2][k] << 16)),
+                             __fsub_rn(rest[2 * k + 1], __uint_as_float(d[2][k] & 0xffff0000u)));
         }
         // (every lane has read all four atoms before the shuffles above)
-        const uint32_t o = atoms + (uint32_t)(g * 1024) + dst;
-        asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(o), "r"(dh[0]), "r"(dh[1]), "r"(dh[2]), "r"(dh[3]) : "memory");
-        asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(o + 512u), "r"(dm[0]), "r"(dm[1]), "r"(dm[2]), "r"(dm[3])
-                     : "memory");
-        asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(lo_atoms + (uint32_t)(g * 512) + dst), "r"(dl[0]), "r"(dl[1]),
-                     "r"(dl[2]), "r"(dl[3])
-                     : "memory");
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const uint32_t o = (i < 2 ? atoms : low_atoms) + (uint32_t)(g * 1024 + (i & 1) * 512) + dst;
+            asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(o), "r"(d[i][0]), "r"(d[i][1]), "r"(d[i][2]), "r"(d[i][3])
+                         : "memory");
+        }
     }
     if (nf) atomicOr(bad, nf);
     return true;
@@ -287,8 +297,8 @@ k_tc_x3(float2 *__restrict__ sv, const __grid_constant__ TcGeom G, const __grid_
         if (threadIdx.x == 0) atomicExch(d_err, kErrSmemAlign);
         return;
     }
-    Ctl &S = *reinterpret_cast<Ctl *>(smem_dyn + kStages * kStage + kGuard);
-    const uint32_t sB0 = smem_u32(smem_dyn);
+    Ctl &S = *reinterpret_cast<Ctl *>(smem_dyn + kStages * kRaw + kLows * kLow + kGuard);
+    const uint32_t sB0 = smem_u32(smem_dyn), sLow0 = sB0 + (uint32_t)(kStages * kRaw);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     volatile int *abort_flag = &S.abort;
 
@@ -298,6 +308,7 @@ k_tc_x3(float2 *__restrict__ sv, const __grid_constant__ TcGeom G, const __grid_
             mbar_init(smem_u32(&S.full[i]), kConvWarps * 32);
             mbar_init(smem_u32(&S.empty[i]), kEpiWarps * 32);
         }
+        for (int i = 0; i < kLows; ++i) mbar_init(smem_u32(&S.low_free[i]), 1);
         mbar_init(smem_u32(&S.acc_full), 1);
         mbar_init(smem_u32(&S.acc_empty), kEpiWarps * 32);
         for (int i = 0; i < 4; ++i) mbar_init(smem_u32(&S.xch[i]), 64);
@@ -349,7 +360,7 @@ k_tc_x3(float2 *__restrict__ sv, const __grid_constant__ TcGeom G, const __grid_
             const int s = i % kStages, n = i / kStages;
             if (n >= 1 && !mbar_wait(smem_u32(&S.empty[s]), (n - 1) & 1, abort_flag, d_err)) break;
             const uint64_t tb = col_base(t * kNT, G);
-            const uint32_t sb = sB0 + (uint32_t)(s * kStage);
+            const uint32_t sb = sB0 + (uint32_t)(s * kRaw);
             if constexpr (TABLE) {
 #pragma unroll 16
                 for (int k = 0; k < 32; ++k) cp_async16(sb + (tsm ^ R.cit_sm[k]), sv + (tb | ta | R.cit_addr[k]), 16u);
@@ -371,9 +382,11 @@ k_tc_x3(float2 *__restrict__ sv, const __grid_constant__ TcGeom G, const __grid_
         for (uint64_t t = blockIdx.x; t < ntl; t += gridDim.x, ++i) {
             const int s = i % kStages;
             if (!mbar_wait(smem_u32(&S.landed[s]), (i / kStages) & 1, abort_flag, d_err)) break;
-            const uint32_t sb = sB0 + (uint32_t)(s * kStage);
-            if (!convert_half<T0>(sb + (uint32_t)(cb * 8192 + half * 4096), sb + (uint32_t)(kRaw + cb * 4096 + half * 2048),
-                                  lane, half, halves, S.share[i & 1][cb], smem_u32(&S.xch[cb]), (uint32_t)(i & 1),
+            const int low = i % kLows;                   // its products of kLows tiles ago are done
+            if (i >= kLows && !mbar_wait(smem_u32(&S.low_free[low]), (i / kLows - 1) & 1, abort_flag, d_err)) break;
+            const uint32_t part = (uint32_t)(cb * 8192 + half * 4096);
+            if (!convert_half<T0>(sB0 + (uint32_t)(s * kRaw) + part, sLow0 + (uint32_t)(low * kLow) + part, lane, half,
+                                  halves, S.share[i & 1][cb], smem_u32(&S.xch[cb]), (uint32_t)(i & 1),
                                   &S.bad[s][half][cb], abort_flag, d_err))
                 break;
             fence_proxy_async();
@@ -386,27 +399,29 @@ k_tc_x3(float2 *__restrict__ sv, const __grid_constant__ TcGeom G, const __grid_
             for (uint64_t t = blockIdx.x; t < ntl; t += gridDim.x, ++i) {
                 const int s = i % kStages;
                 if (!mbar_wait(smem_u32(&S.full[s]), (i / kStages) & 1, abort_flag, d_err)) break;
-                if (i >= 1 && !mbar_wait(smem_u32(&S.acc_empty), (i - 1) & 1, abort_flag, d_err)) break;
                 tc_fence_after();
-                const uint32_t d0 = tmem + kACols, d1 = d0 + 2 * kNT;
-                const uint32_t b = sB0 + (uint32_t)(s * kStage);
+                const uint32_t d0 = tmem + kACols, d1 = d0 + (uint32_t)(2 * kNT * (1 + (i & 1)));
+                const uint32_t b = sB0 + (uint32_t)(s * kRaw);
                 // K = 64 members in 4 steps of 16: A 8 columns per step, B two member groups.
                 // The descriptors of a tile differ in their start address only (bits 0-13, in
                 // units of 16 bytes); one thread issues everything, so each is one addition
-                const uint64_t bhm = sdesc_b(b, 8192u, 1024u), blo = sdesc_b(b + (uint32_t)kRaw, 4096u, 512u);
+                const uint64_t bd = sdesc_b(b, 8192u, 1024u), bl = sdesc_b(sLow0 + (uint32_t)(i % kLows * kLow), 8192u, 1024u);
                 auto step = [&](uint32_t d, int da, int db, int ks, uint32_t acc) {
-                    const uint64_t bd = db < 2 ? bhm + (uint64_t)((ks * 2048 + db * 512) >> 4)
-                                               : blo + (uint64_t)((ks * 1024) >> 4);
-                    mma_bf16(d, tmem + (uint32_t)(da * 32 + ks * 8), bd, acc);
+                    mma_bf16(d, tmem + (uint32_t)(da * 32 + ks * 8),
+                             (db < 2 ? bd : bl) + (uint64_t)((ks * 2048 + (db & 1) * 512) >> 4), acc);
                 };
+                // the smaller products first. Their accumulator was read two tiles ago (the wait
+                // below, one tile ago); the epilogue may still read the tile before
+                constexpr int pa[12] = {3, 2, 1, 3, 2, 1, 0, 2, 1, 0, 1, 0}, pb[12] = {1, 2, 3, 0, 1, 2, 3, 0, 1, 2, 0, 1};
 #pragma unroll
-                for (int ks = 0; ks < 4; ++ks) step(d0, 0, 0, ks, ks);
-                // the smaller products first
-                constexpr int pa[8] = {3, 2, 1, 2, 1, 0, 1, 0}, pb[8] = {0, 1, 2, 0, 1, 2, 0, 1};
-#pragma unroll
-                for (int p = 0; p < 8; ++p)
+                for (int p = 0; p < 12; ++p)
 #pragma unroll
                     for (int ks = 0; ks < 4; ++ks) step(d1, pa[p], pb[p], ks, p + ks);
+                mma_commit(smem_u32(&S.low_free[i % kLows]));
+                if (i >= 1 && !mbar_wait(smem_u32(&S.acc_empty), (i - 1) & 1, abort_flag, d_err)) break;
+                tc_fence_after();
+#pragma unroll
+                for (int ks = 0; ks < 4; ++ks) step(d0, 0, 0, ks, ks);
                 mma_commit(smem_u32(&S.acc_full));
             }
             mma_commit(smem_u32(&S.done));
@@ -435,13 +450,13 @@ k_tc_x3(float2 *__restrict__ sv, const __grid_constant__ TcGeom G, const __grid_
             const int s = i % kStages;
             if (!mbar_wait(smem_u32(&S.acc_full), i & 1, abort_flag, d_err)) break;
             tc_fence_after();
-            const uint32_t sb = sB0 + (uint32_t)(s * kStage);
+            const uint32_t sb = sB0 + (uint32_t)(s * kRaw);
             const uint64_t tb = col_base(t * kNT, G);
 #pragma unroll 1
             for (int cc = 0; cc < 4; ++cc) {
                 float v[16], w[16];
                 const uint32_t ad = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(kACols + hh * kNT + cc * 16);
-                tmem_ld16x2(ad, ad + 2 * kNT, v, w);
+                tmem_ld16x2(ad, ad + (uint32_t)(2 * kNT * (1 + (i & 1))), v, w);
 #pragma unroll
                 for (int k = 0; k < 16; ++k) v[k] += w[k];
                 const int blk = 2 * hh + (cc >> 1);
@@ -523,17 +538,14 @@ std::vector<uint16_t> build_image(const double *g, int k) {
         const double scale = std::ldexp(1.0, 7 - e);
         for (int l = 0; l < D; ++l) t[l] *= scale;       // now in units of the first digit
         for (int d = 0; d < kDigA; ++d) {
-            // multiples of 2^(e - 7 - 8 d); the last digit is what is left, in BF16
-            const float unit = std::ldexp(1.0f, e - 7 - 8 * d);
+            // multiples of 2^(e - 7) and 2^(e - 15), then twice what is left, in BF16
+            const float unit = std::ldexp(1.0f, e - 7 - 8 * std::min(d, 2));
             uint16_t *out = &img[(size_t)(d * 128 + m) * 64 + (j & ~(D - 1))];
             constexpr double kRound = 6755399441055744.0;   // 1.5 2^52: adding it rounds to an integer
             for (int l = 0; l < D; ++l) {
-                const double v = d + 1 < kDigA ? (t[l] + kRound) - kRound : t[l];
-                const float f = (float)v * unit;
-                uint32_t u;
-                std::memcpy(&u, &f, 4);
-                out[l] = (uint16_t)((u + 0x7fffu + ((u >> 16) & 1u)) >> 16);
-                t[l] = (t[l] - v) * 256.0;
+                const double v = d < 2 ? (t[l] + kRound) - kRound : bf16_to_float(host_bf16((float)t[l]));
+                out[l] = host_bf16((float)v * unit);
+                t[l] = (t[l] - v) * (d < 2 ? 256.0 : 1.0);
             }
         }
     }
@@ -559,9 +571,9 @@ cudaError_t run(const LaunchCtx &L, float2 *sv, const TcGeom &G, const RawMap &R
 // are relative to its largest entry and those of a column to its largest
 // amplitude, so a matrix with zero entries -- whose outputs may not see the
 // amplitude that sets the scale -- stays with the FP32 kernels. Random unitaries
-// and states on 20 qubits, relative L2 error against 64 bits: one gate 6.9e-8
-// (k = 5) and 7.7e-8 (k = 6) where the FP32 chains have 1.5e-7, fifty gates
-// 4.8e-7 and 5.4e-7 against 1.04e-6 and 1.05e-6; no drift of the norm.
+// and states on 23 qubits, relative L2 error against 64 bits: one gate 3.7e-8 where
+// the FP32 chains have 1.5e-7 (k = 5 and 6), fifty gates 2.6e-7 against 1.04e-6; no
+// drift of the norm.
 bool tc_x3_ok(int n, int k, const double *mat) {
     if (n < (k == 5 ? 23 : 22) || k < 5 || k > 6) return false;
     int lo = 5000, hi = -5000;
