@@ -566,26 +566,33 @@ cudaError_t run(const LaunchCtx &L, float2 *sv, const TcGeom &G, const RawMap &R
 }  // namespace
 
 // Large states only: a gate's matrix takes the host 22 / 43 us to cut and upload
-// (k = 5 / 6), as long as k_dense5 / k_dense6 take on 22 qubits (33 / 73 us a gate
-// there, 100 / 225 us on 24, against 87 us for either here). The digits of a row
-// are relative to its largest entry and those of a column to its largest
-// amplitude, so a matrix with zero entries -- whose outputs may not see the
-// amplitude that sets the scale -- stays with the FP32 kernels. Random unitaries
-// and states on 23 qubits, relative L2 error against 64 bits: one gate 3.7e-8 where
-// the FP32 chains have 1.5e-7 (k = 5 and 6), fifty gates 2.6e-7 against 1.04e-6; no
-// drift of the norm.
+// (k = 5 / 6). Gates in a row, us each, here and by k_dense5 / k_dense6: k = 5 on 22
+// qubits 42 / 39, 23 58 / 58, 24 90 / 107; k = 6 on 21 qubits 59 / 53, 22 60 / 82,
+// 23 62 / 130.
+//
+// The digits leave out about 2^-34 of a row's largest entry and of a group's largest
+// part per product. An output whose row meets the one large amplitude of its group with
+// a small entry feels this first, so every entry has to be within 2^10 of the largest of
+// its row (and zeros stay with the FP32 kernels): the worst amplitude of adversarial
+// groups then has 4.4 u sum |m||x| in a model of the digits and 6.6 u measured, where a
+// chain of 2 2^k FP32 multiply-adds has up to 22 u; at 2^13 it would have 2.4 times the
+// chain's error. Random unitaries are within 2^10 (99 %). Random unitaries and states on 23
+// qubits, relative L2 error against 64 bits: one gate 3.7e-8 where the FP32 chains have
+// 1.5e-7 (k = 5 and 6), fifty gates 2.6e-7 against 1.04e-6; no drift of the norm.
 bool tc_x3_ok(int n, int k, const double *mat) {
     if (n < (k == 5 ? 23 : 22) || k < 5 || k > 6) return false;
-    int lo = 5000, hi = -5000;
-    for (int i = 0; i < (1 << (2 * k)); ++i) {
-        const double a = std::fmax(std::fabs(mat[2 * i]), std::fabs(mat[2 * i + 1]));
-        if (!std::isfinite(mat[2 * i]) || !std::isfinite(mat[2 * i + 1]) || a == 0.0) return false;
-        int e;
-        std::frexp(a, &e);
-        lo = std::min(lo, e);
-        hi = std::max(hi, e);
+    const int D = 1 << k;
+    for (int r = 0; r < D; ++r) {
+        double lo = HUGE_VAL, hi = 0.0;
+        for (int c = 0; c < D; ++c) {
+            const double *m = mat + 2 * (r * D + c), a = m[0] * m[0] + m[1] * m[1];
+            lo = std::fmin(lo, a);
+            hi = std::fmax(hi, a);
+            if (!std::isfinite(a)) return false;
+        }
+        if (lo * 0x1p20 < hi || lo < 0x1p-120 || hi > 0x1p120) return false;
     }
-    return hi - lo <= 14 && hi <= 60 && lo >= -60;
+    return true;
 }
 
 cudaError_t launch_tc_x3(const LaunchCtx &L, void *sv, int n, const int *tpos, int k, const double *mat, void *d_a,

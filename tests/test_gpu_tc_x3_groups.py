@@ -5,7 +5,10 @@ u = 2^-24, the closing additions round to about 4 u sum |m||x| per amplitude. Th
 2^-34 of the group's largest part and of the row's largest entry per product; over 128 products of random sign
 (rms a third of the most, 4.5 standard deviations) that is 2^-31 of both, 8 u sum |m||x| at the widest row
 spread that the digits serve (an entry 2^-10 of the row's largest that meets the one large amplitude).
-Tolerance per amplitude: 12 u sum |m||x| over the group, and 10 u of the norm per group."""
+Tolerance per amplitude: 12 u sum |m||x| over the group, and 10 u of the norm per group; matrices of a wider spread are
+left to FP32 chains, whose 2 * 2^k partial sums (each at most sum |m||x|) round by u / sqrt(3) rms: 4.5 deviations are
+4.5 sqrt(2 * 2^k / 3) u per amplitude. Where the entries' spread is what is tested, the worst amplitude of 4096 groups
+is also held to twice that of such a chain on the same groups."""
 import numpy as np
 import pytest
 
@@ -18,7 +21,7 @@ TARGETS = [(23, (0, 3, 5, 8, 9)), (23, (1, 3, 5, 8, 9)), (23, (22, 4, 6, 8, 9)),
            (22, (1, 2, 4, 9, 12, 21)), (22, (4, 9, 12, 6, 11, 5))]
 
 
-def check(v, targets, m, parts=False):
+def check(v, targets, m, parts=False, limit=12):
     n = v.size.bit_length() - 1
     v = v.astype(np.complex64)
     at = groups(n, targets)
@@ -30,11 +33,30 @@ def check(v, targets, m, parts=False):
     norm = np.linalg.norm(want, axis=0)
     group = np.max(np.linalg.norm(err, axis=0) / (norm + 1e-35))
     print(f"worst {worst:.2f} u, group {group:.2e}")
-    assert worst <= 12
-    assert group <= 10 * U
+    assert worst <= limit
+    assert group <= 10 * U or limit > 12
     if parts:
         for a, b in ((got.real - want.real, np.abs(x.real)), (got.imag - want.imag, np.abs(x.imag))):
             assert np.all(np.abs(a) <= 12 * U * (np.abs(m.real) @ b) + 1e-40)
+    return x, want, got
+
+
+def chain(k):
+    return 4.5 * (2 * 2 ** k / 3) ** 0.5
+
+
+def fp32_chain(m, x):
+    """The product as one chain of FP32 multiply-adds per part, members in order."""
+    m, x = m.astype(np.complex64), x.astype(np.complex64)
+
+    def fma(a, b, c):
+        return (a.astype(float) * b.astype(float) + c).astype(np.float32)
+
+    re = im = np.zeros((m.shape[0], x.shape[1]), np.float32)
+    for a, b in zip(m.T[:, :, None], x[:, None, :]):
+        re = fma(-a.imag, b.imag, fma(a.real, b.real, re))
+        im = fma(a.imag, b.real, fma(a.real, b.imag, im))
+    return re.astype(float) + 1j * im
 
 
 def lowest_free(targets):
@@ -70,7 +92,7 @@ def limit_matrix(k, spread):
 
 
 @pytest.mark.parametrize("k", [5, 6])
-@pytest.mark.parametrize("spread", [0, 4, 8, 9.999])
+@pytest.mark.parametrize("spread", [0, 4, 8, 9.999, 11, 13])
 def test_one_large_amplitude_meets_the_small_entries(k, spread):
     n, targets = 23, (2, 5, 6, 11, 13, 17)[:k]
     m = gen.random_gate_dense(gen.rng_for(k), k) if spread == 0 else limit_matrix(k, spread)
@@ -78,7 +100,22 @@ def test_one_large_amplitude_meets_the_small_entries(k, spread):
     for depth in (8, 12, 16, 20):
         v = gen.random_state(n, depth) * 2.0 ** (n / 2 - depth)
         v[at[3]] = np.exp(1j * np.arange(at.shape[1]))
-        check(v, targets, m)
+        x, want, got = (a[:, :4096] for a in check(v, targets, m, limit=12 if spread <= 10 else chain(k)))
+        scale = np.abs(m) @ np.abs(x)
+        assert np.max(np.abs(got - want) / scale) <= 2 * np.max(np.abs(fp32_chain(m, x) - want) / scale)
+
+
+@pytest.mark.parametrize("k", [5, 6])
+@pytest.mark.parametrize("angle", [0.01, 0.3])
+def test_near_identity(k, angle):
+    """exp(-i angle H) for a Hermitian H without zero entries, on groups with one large amplitude."""
+    n, targets = 23, (0, 5, 6, 11, 13, 17)[:k]
+    a = gen.random_gate_dense(gen.rng_for(k), k)
+    w, q = np.linalg.eigh(a + a.conj().T)
+    m = (q * np.exp(-1j * angle * w)) @ q.conj().T
+    v = gen.random_state(n, 2) * 2.0 ** (n / 2 - 12)
+    v[groups(n, targets)[1]] = 1
+    check(v, targets, m, limit=chain(k))
 
 
 @pytest.mark.parametrize("k", [5, 6])
