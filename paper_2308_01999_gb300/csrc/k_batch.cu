@@ -641,7 +641,8 @@ __device__ __noinline__ void pauli_group(const float2 *tile, const float2 *sv, b
         }
     }
 #pragma unroll
-    for (int k = 0; k < R; ++k) tot[k] = block_sum(2.0 * ((double)acc[k] + (double)cmp[k]), red);
+    for (int k = 0; k < R; ++k)
+        tot[k] = block_sum(2.0 * ((double)acc[k] + (isfinite(acc[k]) ? (double)cmp[k] : 0.0)), red);   // inf - inf in cmp
 }
 
 // how many of the strings from s on share a pass: 3 or 2 with independent masks, else 1
