@@ -22,6 +22,9 @@
 //               kernel check that entries (dm bits) and nonzero amplitudes (t
 //               bits) lie within t + dm <= 24 bits of their largest, which again
 //               bounds the error by that of FP64 term by term; zeros are exact.
+// What is bounded is the error of an amplitude's modulus. A part far below its
+// amplitude carries that error too, unless the matrix keeps the parts apart (below).
+//
 // A group outside these ranges (also infinities, NaN, values near the limits of
 // the exponent) is computed in FP64 in the same kernel, with k_dense's sums in
 // k_dense's order.
@@ -72,6 +75,30 @@ __device__ __forceinline__ uint64_t mant64(int hi, int lo) {
     return ((uint64_t)(__funnelshift_l((uint32_t)lo, (uint32_t)hi, 11) | 0x80000000u) << 32) | ((uint32_t)lo << 11);
 }
 
+// How a matrix mixes real and imaginary parts. In general every output part sees
+// both and a group has one scale. A matrix that is real once some rows and columns
+// are multiplied by i (real gates, RX) keeps two classes of reals apart: class 0
+// holds the real parts of columns whose bit in col is clear and the imaginary parts
+// of the others, class 1 the rest, and row j's real part sums the class that its bit
+// in row names. Then (SPLIT) each class has a scale of its own, so that small parts
+// beside large ones keep their accuracy, as they do in FP64. 26 qubits, with and
+// without: 0.34 / 0.32 ms for k = 1, 0.47 / 0.45 for k = 2, 0.87 / 0.79 and 1.04 / 0.91
+// for k = 3 and 4, 2.06 / 2.02 for k = 5.
+struct Parts {
+    uint32_t row, col;
+    bool split;
+};
+
+// The classes of an amplitude's parts r, i (and back: a row's parts of the two classes' values)
+template <typename T>
+__device__ __forceinline__ void by_class(uint32_t bits, int l, const T &r, const T &i, T &c0, T &c1) {
+    const bool f = ((bits >> l) & 1u) != 0;
+    c0 = f ? i : r;
+    c1 = f ? r : i;
+}
+
+__device__ __forceinline__ bool out_of_range(int E) { return (unsigned)(E - kEMin) > (unsigned)(kEMax - kEMin); }
+
 // ---------------------------------------------------------------------------
 // two limbs of 30 bits. x = (x1 2^30 + x0) 2^-P 2^(E - 1022), sign and
 // magnitude, P = 60 (k = 1) or 59 (k = 2) bits; m = (m1 2^30 + m0) 2^-PM 2^em
@@ -88,10 +115,11 @@ template <int K> struct Fx2 {
     static constexpr int P = 61 - K, PM = 61 - K;
     int m[1 << (2 * K)][4];         // r1, r0, i1, i0
     int em;
+    Parts parts;
     double2 f[1 << (2 * K)];        // for groups out of range
 };
 
-template <int K, int U>
+template <int K, int U, bool SPLIT>
 __global__ void __launch_bounds__(kThreads, K == 1 ? 4 : 3)
 k_dense_fx2(double2 *__restrict__ sv, uint64_t n_groups, GroupGeom G, Offs<K> O, Fx2<K> M) {
     constexpr int D = 1 << K, P = Fx2<K>::P, PM = Fx2<K>::PM;
@@ -112,42 +140,65 @@ k_dense_fx2(double2 *__restrict__ sv, uint64_t n_groups, GroupGeom G, Offs<K> O,
 #pragma unroll
     for (int u = 0; u < U; ++u) {
         if (u0 + (uint64_t)u * kThreads >= n_groups) continue;
-        int hi[2 * D], lo[2 * D], top = 0;
+        int hi[2 * D], lo[2 * D], top[2] = {0, 0};       // by class; of all reals if not SPLIT
 #pragma unroll
         for (int l = 0; l < D; ++l) {
             hi[2 * l] = __double2hiint(v[u][l].x);
             lo[2 * l] = __double2loint(v[u][l].x);
             hi[2 * l + 1] = __double2hiint(v[u][l].y);
             lo[2 * l + 1] = __double2loint(v[u][l].y);
-            top = max(top, max(hi[2 * l] & 0x7fffffff, hi[2 * l + 1] & 0x7fffffff));
+            const int hr = hi[2 * l] & 0x7fffffff, hj = hi[2 * l + 1] & 0x7fffffff;
+            if constexpr (SPLIT) {
+                int c0, c1;
+                by_class(M.parts.col, l, hr, hj, c0, c1);
+                top[0] = max(top[0], c0);
+                top[1] = max(top[1], c1);
+            } else {
+                top[0] = max(top[0], max(hr, hj));
+            }
         }
-        const int E = top >> 20;
-        if ((unsigned)(E - kEMin) > (unsigned)(kEMax - kEMin)) {
-            uint32_t any = 0;
+        int E[2] = {top[0] >> 20, SPLIT ? top[1] >> 20 : top[0] >> 20};
+        if (out_of_range(E[0]) || (SPLIT && out_of_range(E[1]))) {
+            // zeros take any scale; what else is out of range goes to FP64
+            uint32_t any[2] = {0, 0};
 #pragma unroll
-            for (int i = 0; i < 2 * D; ++i) any |= (uint32_t)(hi[i] & 0x7fffffff) | (uint32_t)lo[i];
+            for (int l = 0; l < D; ++l) {
+                const uint32_t ar = (uint32_t)(hi[2 * l] & 0x7fffffff) | (uint32_t)lo[2 * l];
+                const uint32_t aj = (uint32_t)(hi[2 * l + 1] & 0x7fffffff) | (uint32_t)lo[2 * l + 1];
+                if constexpr (SPLIT) {
+                    uint32_t c0, c1;
+                    by_class(M.parts.col, l, ar, aj, c0, c1);
+                    any[0] |= c0;
+                    any[1] |= c1;
+                } else {
+                    any[0] |= ar | aj;
+                }
+            }
+            if ((any[0] && out_of_range(E[0])) || (SPLIT && any[1] && out_of_range(E[1]))) {
 #pragma unroll
-            for (int j = 0; j < D; ++j) {
-                double2 acc = make_double2(0.0, 0.0);
-                if (any) {
+                for (int j = 0; j < D; ++j) {
+                    double2 acc = make_double2(0.0, 0.0);
 #pragma unroll
                     for (int l = 0; l < D; ++l) cmad(acc, M.f[j * D + l], v[u][l]);
+                    sv[base[u] + O.o[j]] = acc;
                 }
-                sv[base[u] + O.o[j]] = acc;
+                continue;
             }
-            continue;
+            if (!any[0]) E[0] = kEMin;
+            if (!SPLIT || !any[1]) E[1] = kEMin;
         }
         int x1[2 * D], x0[2 * D];
 #pragma unroll
         for (int i = 0; i < 2 * D; ++i) {
             const int e = (hi[i] >> 20) & 0x7ff;
-            const uint64_t F = shr64(mant64(hi[i], lo[i]), (uint32_t)(64 - P + E - e));
+            const int Ei = SPLIT && (((M.parts.col >> (i / 2)) ^ i) & 1u) ? E[1] : E[0];
+            const uint64_t F = shr64(mant64(hi[i], lo[i]), (uint32_t)(64 - P + Ei - e));
             const int sg = (hi[i] >> 31) | 1;
             x1[i] = (int)__funnelshift_r((uint32_t)F, (uint32_t)(F >> 32), 30) * sg;
             x0[i] = (int)((uint32_t)F & 0x3fffffffu) * sg;
         }
-        const int sc = E - 1022 + M.em + 60 - P - PM;
-        auto out = [&](long long a1, long long a0) {
+        const int sc[2] = {E[0] - 1022 + M.em + 60 - P - PM, E[1] - 1022 + M.em + 60 - P - PM};
+        auto out = [&](long long a1, long long a0, int sc) {
             return scaled(__ll2double_rn(a1 + ((a0 + (1ll << 29)) >> 30)), sc);
         };
 #pragma unroll
@@ -170,7 +221,9 @@ k_dense_fx2(double2 *__restrict__ sv, uint64_t n_groups, GroupGeom G, Offs<K> O,
                 i0 = mad_wide(b1, m[1], i0);
                 i0 = mad_wide(b0, m[0], i0);
             }
-            sv[base[u] + O.o[j]] = make_double2(out(r1, r0), out(i1, i0));
+            int sr = sc[0], si = sc[0];
+            if constexpr (SPLIT) by_class(M.parts.row, j, sc[0], sc[1], sr, si);
+            sv[base[u] + O.o[j]] = make_double2(out(r1, r0, sr), out(i1, i0, si));
         }
     }
 }
@@ -195,7 +248,8 @@ constexpr int kFx3Threads = 128;
 template <int K> struct Fx3 {
     int m[1 << (2 * K)][6];          // r2, r1, r0, i2, i1, i0
     int em;
-    int t;                           // nonzero amplitudes must lie within 2^t of the largest
+    int t;                           // nonzero amplitudes (SPLIT: reals of a class) must lie within 2^t of the largest
+    Parts parts;
     double2 f[1 << (2 * K)];
 };
 
@@ -229,7 +283,7 @@ __device__ __forceinline__ double out3(long long a2, long long a1, long long a0,
 // A group is shared by S lanes, DL = 2^K / S of its amplitudes each (lane s holds
 // members s DL .. s DL + DL - 1): each lane sums its members' share of S rows,
 // then hands every other lane its row's partial sums and finishes one row.
-template <int K, int S>
+template <int K, int S, bool SPLIT>
 __global__ void __launch_bounds__(kFx3Threads, 4)
 k_dense_fx3(double2 *__restrict__ sv, uint64_t n_groups, GroupGeom G, const __grid_constant__ Offs<K> O,
             const __grid_constant__ Fx3<K> M) {
@@ -249,38 +303,61 @@ k_dense_fx3(double2 *__restrict__ sv, uint64_t n_groups, GroupGeom G, const __gr
     const uint64_t base = insert_zeros(g, G);
     wait_for_previous();
     int x[2 * DL][3];
-    int E;
+    constexpr int NC = SPLIT ? 2 : 1;                   // scales
+    int E[NC];
     bool slow, zero;
     {
         double2 v[DL];
 #pragma unroll
         for (int j = 0; j < DL; ++j) v[j] = sv[base + O.o[s * DL + j]];
-        int top = 0;
-        uint32_t low = 0xffffffffu, denorm = 0;
+        int top[NC];
+        uint32_t low[NC], denorm = 0;
+#pragma unroll
+        for (int c = 0; c < NC; ++c) {
+            top[c] = 0;
+            low[c] = 0xffffffffu;
+        }
 #pragma unroll
         for (int l = 0; l < DL; ++l) {
             const int hr = __double2hiint(v[l].x) & 0x7fffffff, hj = __double2hiint(v[l].y) & 0x7fffffff;
-            const uint32_t lw = (uint32_t)__double2loint(v[l].x) | (uint32_t)__double2loint(v[l].y);
-            const int a = max(hr, hj);
-            top = max(top, a);
-            low = min(low, (uint32_t)a - 1u);          // an exact zero wraps around and does not count
-            if (a == 0) denorm |= lw;
+            const uint32_t lr = (uint32_t)__double2loint(v[l].x), lj = (uint32_t)__double2loint(v[l].y);
+            int a[NC];
+            if constexpr (SPLIT) {
+                by_class(M.parts.col, s * DL + l, hr, hj, a[0], a[NC - 1]);
+                if (hr == 0) denorm |= lr;
+                if (hj == 0) denorm |= lj;
+            } else {
+                a[0] = max(hr, hj);
+                if (a[0] == 0) denorm |= lr | lj;
+            }
+#pragma unroll
+            for (int c = 0; c < NC; ++c) {
+                top[c] = max(top[c], a[c]);
+                low[c] = min(low[c], (uint32_t)a[c] - 1u);   // an exact zero wraps around and does not count
+            }
         }
 #pragma unroll
         for (int o = 1; o < S; o <<= 1) {
-            top = max(top, __shfl_xor_sync(0xffffffffu, top, o));
-            low = min(low, __shfl_xor_sync(0xffffffffu, low, o));
+#pragma unroll
+            for (int c = 0; c < NC; ++c) {
+                top[c] = max(top[c], __shfl_xor_sync(0xffffffffu, top[c], o));
+                low[c] = min(low[c], __shfl_xor_sync(0xffffffffu, low[c], o));
+            }
             denorm |= __shfl_xor_sync(0xffffffffu, denorm, o);
         }
-        E = top >> 20;
-        zero = ((uint32_t)top | denorm) == 0;           // the product of zeros: the amplitudes stay zero
-        slow = !zero && ((unsigned)(E - kEMin) > (unsigned)(kEMax - kEMin) || denorm != 0 ||
-                         (uint32_t)top - low > ((uint32_t)M.t << 20));
+        zero = ((uint32_t)(top[0] | top[NC - 1]) | denorm) == 0;   // the product of zeros: the amplitudes stay zero
+        slow = denorm != 0;
+#pragma unroll
+        for (int c = 0; c < NC; ++c) {
+            slow = slow || (uint32_t)top[c] - low[c] > ((uint32_t)M.t << 20) || (top[c] != 0 && out_of_range(top[c] >> 20));
+            E[c] = top[c] != 0 ? top[c] >> 20 : kEMin;  // zeros take any scale
+        }
 #pragma unroll
         for (int i = 0; i < 2 * DL; ++i) {
             const double w = (i & 1) ? v[i >> 1].y : v[i >> 1].x;
             const int hi = __double2hiint(w);
-            const uint32_t d = (uint32_t)(E - ((hi >> 20) & 0x7ff));
+            const int Ei = SPLIT && (((M.parts.col >> (s * DL + (i >> 1))) ^ i) & 1u) ? E[NC - 1] : E[0];
+            const uint32_t d = (uint32_t)(Ei - ((hi >> 20) & 0x7ff));
             const uint64_t m = mant64(hi, __double2loint(w));
             const uint64_t hl = shr64(m, d);
             const uint32_t r2 = (uint32_t)(hl >> 32), r1 = (uint32_t)hl;
@@ -315,7 +392,7 @@ k_dense_fx3(double2 *__restrict__ sv, uint64_t n_groups, GroupGeom G, const __gr
     const bool store = valid && !slow && !zero;
     // weight of a2: 2^(4L - 84 - 83 + E - 1022 + em); its bit 63 has biased exponent
     // that plus 63 + 1023
-    const int be = E + M.em + 64 + 4 * kL - 167;
+    const int be[2] = {E[0] + M.em + 64 + 4 * kL - 167, E[NC - 1] + M.em + 64 + 4 * kL - 167};
     // the row loop stays rolled (the unrolled kernel would not fit the instruction cache)
 #pragma unroll 1
     for (int j = 0; j < D; j += S) {
@@ -372,7 +449,9 @@ k_dense_fx3(double2 *__restrict__ sv, uint64_t n_groups, GroupGeom G, const __gr
                 trade(im[r].a0, im[r + o].a0);
             }
         }
-        const double2 w = make_double2(out3(re[0].a2, re[0].a1, re[0].a0, be), out3(im[0].a2, im[0].a1, im[0].a0, be));
+        int br = be[0], bi = be[0];
+        if constexpr (SPLIT) by_class(M.parts.row, j + s, be[0], be[1], br, bi);
+        const double2 w = make_double2(out3(re[0].a2, re[0].a1, re[0].a0, br), out3(im[0].a2, im[0].a1, im[0].a0, bi));
         if (store) sv[base + O.o[j + s]] = w;
     }
 }
@@ -418,6 +497,7 @@ template <int K> struct Fxt {
     long long m[1 << (2 * K)][2];   // round(2^(P - em) re, im)
     double2 f[1 << (2 * K)];        // for groups out of range
     int em;
+    Parts parts;
 };
 
 // digit i (from the top) of the offset fixed-point numbers r, j as two FP16 integers
@@ -444,7 +524,7 @@ __device__ __forceinline__ void mma16816(float (&c)[4], const uint4 &a, uint32_t
                  : "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b0), "r"(b1));
 }
 
-template <int K>
+template <int K, bool SPLIT>
 __global__ void __launch_bounds__(kFxtThreads, FxtCfg<K>::blocks)
 k_dense_fxt(double2 *__restrict__ sv, uint64_t n_groups, GroupGeom G, const __grid_constant__ Offs<K> O,
             const Fxt<K> *__restrict__ Mg, const __grid_constant__ Fxt<(K <= 4 ? K : 1)> Mp) {
@@ -459,6 +539,7 @@ k_dense_fxt(double2 *__restrict__ sv, uint64_t n_groups, GroupGeom G, const __gr
     let_next_start();
     if constexpr (K > 4) wait_for_previous();          // the matrix is in the workspace
     const int em = K <= 4 ? Mp.em : Mg->em;
+    const uint32_t prow = K <= 4 ? Mp.parts.row : Mg->parts.row, pcol = K <= 4 ? Mp.parts.col : Mg->parts.col;
     // A's fragments: lane 4 r + q holds rows r (re of member r) and r + 8 (its im),
     // members q (registers x, y) and q + 4 (z, w) of the step
     for (int i = threadIdx.x; i < TM * TM * 32; i += kFxtThreads) {
@@ -493,40 +574,58 @@ k_dense_fxt(double2 *__restrict__ sv, uint64_t n_groups, GroupGeom G, const __gr
         const bool valid = t * 8 + gcol < n_groups;
         const uint64_t base = next;
         uint32_t b[NA][ND];
-        int E;
+        constexpr int NC = SPLIT ? 2 : 1;               // scales
+        int E[NC];
         bool slow, zero;
         {
-            int top = 0;
-            uint32_t any = 0;
+            int top[NC];
+            uint32_t any = 0;                           // low words (SPLIT: of reals whose upper word is zero)
+#pragma unroll
+            for (int c = 0; c < NC; ++c) top[c] = 0;
+            auto upper = [&](int i, int (&a)[NC]) {     // an amplitude's magnitude, or its classes'
+                const int hr = __double2hiint(v[i].x) & 0x7fffffff, hj = __double2hiint(v[i].y) & 0x7fffffff;
+                if constexpr (SPLIT) by_class(pcol, 4 * i + q, hr, hj, a[0], a[NC - 1]);
+                else a[0] = max(hr, hj);
+            };
 #pragma unroll
             for (int i = 0; i < NA; ++i) {
-                const int hr = __double2hiint(v[i].x) & 0x7fffffff, hj = __double2hiint(v[i].y) & 0x7fffffff;
-                top = max(top, max(hr, hj));
-                any |= (uint32_t)__double2loint(v[i].x) | (uint32_t)__double2loint(v[i].y);
+                int a[NC];
+                upper(i, a);
+#pragma unroll
+                for (int c = 0; c < NC; ++c) top[c] = max(top[c], a[c]);
+                if (!SPLIT || (__double2hiint(v[i].x) & 0x7fffffff) == 0) any |= (uint32_t)__double2loint(v[i].x);
+                if (!SPLIT || (__double2hiint(v[i].y) & 0x7fffffff) == 0) any |= (uint32_t)__double2loint(v[i].y);
             }
 #pragma unroll
             for (int o = 1; o < 4; o <<= 1) {
-                top = max(top, __shfl_xor_sync(0xffffffffu, top, o));
+#pragma unroll
+                for (int c = 0; c < NC; ++c) top[c] = max(top[c], __shfl_xor_sync(0xffffffffu, top[c], o));
                 any |= __shfl_xor_sync(0xffffffffu, any, o);
             }
-            E = top >> 20;
-            zero = ((uint32_t)top | any) == 0;
-            slow = !zero && (unsigned)(E - kEMin) > (unsigned)(kEMax - kEMin);
+            zero = ((uint32_t)(top[0] | top[NC - 1]) | any) == 0;
+            slow = SPLIT && any != 0;
+#pragma unroll
+            for (int c = 0; c < NC; ++c) {
+                slow = slow || ((SPLIT ? top[c] != 0 : !zero) && out_of_range(top[c] >> 20));
+                E[c] = top[c] != 0 ? top[c] >> 20 : kEMin;   // zeros take any scale
+            }
 #pragma unroll
             for (int i = 0; i < NA; ++i) {
-                auto fixed = [&](double w) {
+                auto fixed = [&](double w, int e) {
                     const int hi = __double2hiint(w);
-                    const uint64_t F = shr64(mant64(hi, __double2loint(w)), (uint32_t)(64 - P + E - ((hi >> 20) & 0x7ff)));
+                    const uint64_t F = shr64(mant64(hi, __double2loint(w)), (uint32_t)(64 - P + e - ((hi >> 20) & 0x7ff)));
                     return hi < 0 ? off - F : off + F;
                 };
-                const uint64_t fr = fixed(v[i].x), fj = fixed(v[i].y);
+                int er = E[0], ej = E[0];
+                if constexpr (SPLIT) by_class(pcol, 4 * i + q, E[0], E[NC - 1], er, ej);
+                const uint64_t fr = fixed(v[i].x, er), fj = fixed(v[i].y, ej);
 #pragma unroll
                 for (int d = 0; d < ND; ++d) b[i][d] = digits<ND, B>(fr, fj, d);
             }
         }
         bool store = valid && !slow && !zero;
         if (__any_sync(0xffffffffu, slow)) {
-            // a group outside the exponent range: lane q computes rows q NA .. q NA + NA - 1 in FP64
+            // a group outside the range: lane q computes rows q NA .. q NA + NA - 1 in FP64
             double2 acc[NA];
 #pragma unroll
             for (int j = 0; j < NA; ++j) acc[j] = make_double2(0.0, 0.0);
@@ -547,13 +646,14 @@ k_dense_fxt(double2 *__restrict__ sv, uint64_t n_groups, GroupGeom G, const __gr
         if (t + step < n_tiles) load(t + step);
         // what the output lanes need of columns 2 q and 2 q + 1
         uint64_t ob[2];
-        int sc[2];
+        int sc[2][NC];
         bool st[2];
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             const int from = 4 * (2 * q + h);
             ob[h] = __shfl_sync(0xffffffffu, base, from);
-            sc[h] = __shfl_sync(0xffffffffu, E, from) - 1022 + em - 2 * P + B * (ND - 2);
+#pragma unroll
+            for (int c = 0; c < NC; ++c) sc[h][c] = __shfl_sync(0xffffffffu, E[c], from) - 1022 + em - 2 * P + B * (ND - 2);
             st[h] = __shfl_sync(0xffffffffu, (int)store, from) != 0;
         }
 #pragma unroll 1
@@ -574,7 +674,7 @@ k_dense_fxt(double2 *__restrict__ sv, uint64_t n_groups, GroupGeom G, const __gr
             }
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
-                auto out = [&](int e) {
+                auto out = [&](int e, int shift) {
                     int w[NL];
 #pragma unroll
                     for (int p = 0; p < NL; ++p) w[p] = __float2int_rn(a[p][e]);     // exact: |a| <= 2^24
@@ -589,9 +689,11 @@ k_dense_fxt(double2 *__restrict__ sv, uint64_t n_groups, GroupGeom G, const __gr
                     // per real kept it 75 % busy)
                     const int h1 = (int)(hi >> 32);
                     const int cut = max(0, S + 2 - __clz(h1 ^ (h1 >> 31)));
-                    return scaled(__ll2double_rn((hi << (S - cut)) + (lo >> cut)), sc[h] + cut);
+                    return scaled(__ll2double_rn((hi << (S - cut)) + (lo >> cut)), shift + cut);
                 };
-                const double2 w = make_double2(out(h), out(2 + h));
+                int sr = sc[h][0], si = sc[h][0];
+                if constexpr (SPLIT) by_class(prow, mt * 8 + c, sc[h][0], sc[h][NC - 1], sr, si);
+                const double2 w = make_double2(out(h, sr), out(2 + h, si));
                 if (st[h]) sv[ob[h] + O.o[mt * 8 + c]] = w;
             }
         }
@@ -648,6 +750,45 @@ int take_limb(__int128 &v, int bits) {
     return (int)lo;
 }
 
+// Real up to factors i of rows and columns? (Entries without an imaginary part join a
+// row and a column of equal factors, entries without a real part of different ones.)
+Parts parts_of(const double *mat, int k) {
+    const int D = 1 << k;
+    int row[32], col[32];
+    for (int j = 0; j < D; ++j) row[j] = col[j] = -1;
+    auto kind = [&](int j, int l) {                  // -1: zero, 0 real, 1 imaginary, 2 both
+        const bool r = mat[2 * (j * D + l)] != 0.0, i = mat[2 * (j * D + l) + 1] != 0.0;
+        return r ? (i ? 2 : 0) : (i ? 1 : -1);
+    };
+    for (int j = 0; j < D; ++j) {
+        if (row[j] >= 0) continue;
+        row[j] = 0;
+        int todo[64], n = 0;                         // rows 0 .. 31, columns 32 .. 63
+        todo[n++] = j;
+        while (n > 0) {
+            const int at = todo[--n];
+            for (int o = 0; o < D; ++o) {
+                const int t = at < 32 ? kind(at, o) : kind(o, at - 32);
+                if (t < 0) continue;
+                if (t == 2) return Parts{0, 0, false};
+                int &mine = at < 32 ? row[at] : col[at - 32], &other = at < 32 ? col[o] : row[o];
+                if (other < 0) {
+                    other = mine ^ t;
+                    todo[n++] = at < 32 ? 32 + o : o;
+                } else if (other != (mine ^ t)) {
+                    return Parts{0, 0, false};
+                }
+            }
+        }
+    }
+    Parts p{0, 0, true};
+    for (int j = 0; j < D; ++j) {
+        p.row |= (uint32_t)(row[j] == 1) << j;
+        p.col |= (uint32_t)(col[j] == 1) << j;
+    }
+    return p;
+}
+
 template <int K> void offsets(const int *tpos, Offs<K> &O) {
     for (int j = 0; j < (1 << K); ++j) {
         uint64_t o = 0;
@@ -665,6 +806,7 @@ cudaError_t run_fx2(const LaunchCtx &L, void *sv, uint64_t n_groups, const Group
     offsets<K>(tpos, O);
     Fx2<K> M;
     M.em = em;
+    M.parts = parts_of(mat, K);
     for (int i = 0; i < (1 << (2 * K)); ++i) {
         for (int c = 0; c < 2; ++c) {
             __int128 v = to_fixed(mat[2 * i + c], em, Fx2<K>::PM);
@@ -675,7 +817,8 @@ cudaError_t run_fx2(const LaunchCtx &L, void *sv, uint64_t n_groups, const Group
     }
     const uint64_t per = (uint64_t)kThreads * U;
     ++*L.launches;
-    return launch_dependent(k_dense_fx2<K, U>, (unsigned)((n_groups + per - 1) / per), kThreads, 0, L.stream,
+    return launch_dependent(M.parts.split ? k_dense_fx2<K, U, true> : k_dense_fx2<K, U, false>,
+                            (unsigned)((n_groups + per - 1) / per), kThreads, 0, L.stream,
                             reinterpret_cast<double2 *>(sv), n_groups, G, O, M);
 }
 
@@ -687,6 +830,7 @@ cudaError_t run_fx3(const LaunchCtx &L, void *sv, uint64_t n_groups, const Group
     Fx3<K> M;
     M.em = r.em;
     M.t = 24 - r.dm;
+    M.parts = parts_of(mat, K);
     for (int i = 0; i < (1 << (2 * K)); ++i) {
         for (int c = 0; c < 2; ++c) {
             __int128 v = to_fixed(mat[2 * i + c], r.em, 3 * kL - 1);
@@ -698,24 +842,26 @@ cudaError_t run_fx3(const LaunchCtx &L, void *sv, uint64_t n_groups, const Group
     }
     constexpr int S = K >= 4 ? 2 : 1;
     ++*L.launches;
-    return launch_dependent(k_dense_fx3<K, S>, (unsigned)((n_groups * S + kFx3Threads - 1) / kFx3Threads), kFx3Threads,
-                            0, L.stream, reinterpret_cast<double2 *>(sv), n_groups, G, O, M);
+    return launch_dependent(M.parts.split ? k_dense_fx3<K, S, true> : k_dense_fx3<K, S, false>,
+                            (unsigned)((n_groups * S + kFx3Threads - 1) / kFx3Threads), kFx3Threads, 0, L.stream, reinterpret_cast<double2 *>(sv), n_groups, G, O, M);
 }
 
 template <int K>
 cudaError_t run_fxt(const LaunchCtx &L, void *sv, uint64_t n_groups, const GroupGeom &G, const int *tpos,
-                    const double *mat, int em, void *d_mat) {
+                    const double *mat, const MatRange &r, void *d_mat) {
     using Cfg = FxtCfg<K>;
     Offs<K> O;
     offsets<K>(tpos, O);
+    const Parts parts = parts_of(mat, K);
     auto fill = [&](auto &M) {
-        M.em = em;
+        M.em = r.em;
+        M.parts = parts;
         for (int i = 0; i < (1 << (2 * K)); ++i) {
-            for (int c = 0; c < 2; ++c) M.m[i][c] = (long long)to_fixed(mat[2 * i + c], em, Cfg::P);
+            for (int c = 0; c < 2; ++c) M.m[i][c] = (long long)to_fixed(mat[2 * i + c], r.em, Cfg::P);
             M.f[i] = make_double2(mat[2 * i], mat[2 * i + 1]);
         }
     };
-    auto kern = k_dense_fxt<K>;
+    auto kern = parts.split ? k_dense_fxt<K, true> : k_dense_fxt<K, false>;
     cudaError_t e = cudaSuccess;
     if constexpr (Cfg::smem > 48 * 1024) {
         e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::smem);
@@ -758,9 +904,9 @@ bool try_dense_fx(const LaunchCtx &L, void *sv, int n, const GroupGeom &G, const
         return true;
     }
     if (k >= 3 && !r.zeros && r.dm <= (k == 5 ? 11 : 8)) {
-        e = k == 3   ? run_fxt<3>(L, sv, n_groups, G, tpos, mat, r.em, d_mat)
-            : k == 4 ? run_fxt<4>(L, sv, n_groups, G, tpos, mat, r.em, d_mat)
-                     : run_fxt<5>(L, sv, n_groups, G, tpos, mat, r.em, d_mat);
+        e = k == 3   ? run_fxt<3>(L, sv, n_groups, G, tpos, mat, r, d_mat)
+            : k == 4 ? run_fxt<4>(L, sv, n_groups, G, tpos, mat, r, d_mat)
+                     : run_fxt<5>(L, sv, n_groups, G, tpos, mat, r, d_mat);
         return true;
     }
     if (k > 4 || r.dm > 16) return false;
