@@ -10,24 +10,32 @@
 // products are summed in 64-bit integers (no rounding, no overflow: the bounds
 // are with the layouts below), and each sum is rounded once to a double.
 //
-// Two layouts:
-//   two limbs   k = 1, 2: 3 limb products per real product. Errors are below
-//               about 2^-58 X max|m| 2^k, X the group's largest amplitude, so
-//               the host uses it where every entry is within 2^6 (k = 1) or 2^5
-//               (k = 2) of the largest: then every output holds a term
-//               |m||x| >= 2^-6 max|m| X, and the error stays below the FP64
-//               kernel's own bound 2^-53 sum |m||x| whatever the data.
-//   three limbs 6 limb products per real product (complex products by three
-//               real ones, exact in integers): about 84 bits. The host and the
-//               kernel check that entries (dm bits) and nonzero amplitudes (t
-//               bits) lie within t + dm <= 24 bits of their largest, which again
-//               bounds the error by that of FP64 term by term; zeros are exact.
+// Three layouts (u = 2^-53, X a group's largest amplitude; dm: the bits by which the
+// smallest nonzero entry's exponent lies below the largest's):
+//   two limbs   k = 1, 2: 60 and 59 bits, 3 limb products per real product.
+//   digits      k = 3 to 5: 61 and 62 bits, on the tensor cores.
+//   three limbs k = 1 to 4: 84 bits, 6 limb products per real product (complex
+//               products by three real ones, exact in integers).
+// The first two hold an amplitude to a fixed share of X, so a sum that sees X only
+// through a small entry is less accurate than one that sees it through a large one.
+// Their ranges of dm are those in which the worst amplitude of adversarial groups (the
+// smallest entries on the large amplitudes) has no larger an error, in u sum |m||x|,
+// than a chain of FP64 multiply-adds on the same groups; worst measured here / chain:
+//   k = 1, dm 5: 2.5 / 3.0   k = 2, dm 4: 3.7 / 4.8   (k = 2 at 5: 9.5 / 4.8)
+//   k = 3, dm 7: 5.3 / 7.1   k = 4, dm 7: 8.9 / 9.9   k = 5, dm 8: 12.0 / 14.2
+// Beyond that, up to 8 (k = 5: 11), the digits serve groups in which more amplitudes
+// are large than any row has small entries; then every sum sees a large one through a
+// large entry. Three limbs: host and kernel check that entries (dm bits) and nonzero
+// amplitudes (t bits) lie within t + dm <= 24 bits of their largest, which keeps the
+// error of every term below u / 16 of it. Zeros are exact throughout.
+//
 // What is bounded is the error of an amplitude's modulus. A part far below its
 // amplitude carries that error too, unless the matrix keeps the parts apart (below).
 //
 // A group outside these ranges (also infinities, NaN, values near the limits of
 // the exponent) is computed in FP64 in the same kernel, with k_dense's sums in
 // k_dense's order.
+#include <algorithm>
 #include <cmath>
 #include <vector>
 
@@ -238,8 +246,8 @@ k_dense_fx2(double2 *__restrict__ sv, uint64_t n_groups, GroupGeom G, Offs<K> O,
 //
 // What bounds it: the integer multiply-adds (18 per complex product; one
 // thread holds a group of up to 16 amplitudes in limbs, the matrix is
-// broadcast from shared memory, 24 bytes per complex product). 26 qubits: 1.02 ms
-// for k = 2 (FP64 2.03), 2.98 for k = 4 (FP64 8.1; four lanes a group or other
+// broadcast from shared memory, 24 bytes per complex product). 26 qubits: 0.79 ms
+// for k = 1 (FP64 1.03), 0.99 for k = 2 (2.05), 1.59 for k = 3 (4.08), 2.98 for k = 4 (8.1; four lanes a group or other
 // occupancies up to 3.46).
 // ---------------------------------------------------------------------------
 constexpr int kL = 28;
@@ -457,13 +465,14 @@ k_dense_fx3(double2 *__restrict__ sv, uint64_t n_groups, GroupGeom G, const __gr
 }
 
 // ---------------------------------------------------------------------------
-// k = 3, 4, 5 on the tensor cores, for matrices with no zero entry and entries within
-// 2^8 of the largest (then, as for two limbs, no range has to be checked in the
-// state). Fixed point of P bits in ND balanced digits of B bits, held as FP16
+// k = 3, 4, 5 on the tensor cores, for matrices with no zero entry. Fixed point of P bits, rounded (truncated, the worst
+// amplitude had twice the error), in ND balanced digits of B bits, held as FP16
 // integers; a group's 2 2^k reals are one column of an mma.sync B operand, the
 // matrix (real 2 x 2 blocks) is A, and digit products of equal weight are summed
 // by the FP32 accumulators, exactly: |digit| <= 2^(B-1), so a sum of 2 2^k terms
-// and up to ND digit pairs stays within 2^24:
+// and up to ND digit pairs stays within 2^24, where every integer is an FP32 number
+// (that the accumulation then rounds nothing is not documented; full sums of largest
+// digits are among the tests):
 //   k = 3, 4: 7 digits of 9 bits, 2^16 * 32 * 7 = 2^23.8
 //   k = 5:    8 digits of 8 bits, 2^14 * 64 * 8 = 2^23
 // Products of digits i, j (from the top) with i + j > ND are left out: below
@@ -480,10 +489,11 @@ k_dense_fx3(double2 *__restrict__ sv, uint64_t n_groups, GroupGeom G, const __gr
 // What bounds it: conversions to digits and back (about 110 instructions per
 // amplitude; ALU 46 %, FP64 25 % busy at k = 4) and the MMAs (53 %), which the 16 to
 // 24 warps of an SM overlap in part; the 32 bytes an amplitude moves are a third to a
-// half of the time. 26 qubits: 0.75 ms for k = 3, 0.90 for k = 4, 2.0 for k = 5 (FP64
-// 4.06, 8.1, 14.0; three limbs 2.98 at k = 4). Three blocks per SM at k = 4: 1.01.
+// half of the time. 26 qubits: 0.79 ms for k = 3, 0.91 for k = 4, 2.0 for k = 5 (FP64
+// 4.08, 8.1, 14.0; three limbs 1.59 and 2.98). Three blocks per SM at k = 4: 1.01.
 // ---------------------------------------------------------------------------
 constexpr int kFxtThreads = 256;
+constexpr int kLarge = 2;                     // an amplitude within 2^kLarge of its group's largest is large
 
 template <int K> struct FxtCfg {
     static constexpr int D = 1 << K, ND = K <= 4 ? 7 : 8, B = K <= 4 ? 9 : 8;
@@ -497,13 +507,15 @@ template <int K> struct Fxt {
     long long m[1 << (2 * K)][2];   // round(2^(P - em) re, im)
     double2 f[1 << (2 * K)];        // for groups out of range
     int em;
+    int few;                        // a row's small entries, at most: as many large amplitudes do not bound every sum
     Parts parts;
 };
 
-// digit i (from the top) of the offset fixed-point numbers r, j as two FP16 integers
-template <int ND, int B>
+// digit i (from the top) of the offset fixed-point numbers r, j as two FP16 integers;
+// HALF: of numbers with one more bit, which is dropped
+template <int ND, int B, int HALF = 0>
 __device__ __forceinline__ uint32_t digits(uint64_t r, uint64_t j, int i) {
-    const int sh = B * (ND - 1 - i);
+    const int sh = B * (ND - 1 - i) + HALF;
     const uint32_t a = (uint32_t)(r >> sh), b = (uint32_t)(j >> sh);
     constexpr uint32_t mask = ((1u << B) - 1u) * 0x00010001u;
     uint32_t p = (__byte_perm(a, b, 0x5410) & mask) | 0x64006400u;        // 1024 + digit + 2^(B-1)
@@ -531,6 +543,7 @@ k_dense_fxt(double2 *__restrict__ sv, uint64_t n_groups, GroupGeom G, const __gr
     using Cfg = FxtCfg<K>;
     constexpr int D = Cfg::D, ND = Cfg::ND, B = Cfg::B, P = Cfg::P, TM = Cfg::TM, NA = D / 4;
     constexpr int NL = ND + 1;                        // levels: digit pairs i + j = 0 .. ND
+    constexpr int HALF = ND * B < 64 ? 1 : 0;
     constexpr uint64_t off = digit_offset<ND, B>();
     extern __shared__ __align__(16) uint4 As[];       // [mt][ks][digit][lane]
     const int lane = threadIdx.x & 31, q = lane & 3, c = lane >> 2;
@@ -538,7 +551,7 @@ k_dense_fxt(double2 *__restrict__ sv, uint64_t n_groups, GroupGeom G, const __gr
     const double2 *Mf = K <= 4 ? reinterpret_cast<const double2 *>(Mp.f) : Mg->f;
     let_next_start();
     if constexpr (K > 4) wait_for_previous();          // the matrix is in the workspace
-    const int em = K <= 4 ? Mp.em : Mg->em;
+    const int em = K <= 4 ? Mp.em : Mg->em, few = K <= 4 ? Mp.few : Mg->few;
     const uint32_t prow = K <= 4 ? Mp.parts.row : Mg->parts.row, pcol = K <= 4 ? Mp.parts.col : Mg->parts.col;
     // A's fragments: lane 4 r + q holds rows r (re of member r) and r + 8 (its im),
     // members q (registers x, y) and q + 4 (z, w) of the step
@@ -609,18 +622,37 @@ k_dense_fxt(double2 *__restrict__ sv, uint64_t n_groups, GroupGeom G, const __gr
                 slow = slow || ((SPLIT ? top[c] != 0 : !zero) && out_of_range(top[c] >> 20));
                 E[c] = top[c] != 0 ? top[c] >> 20 : kEMin;   // zeros take any scale
             }
+            if (few) {
+                // large amplitudes (or reals of a class), in a half-word each
+                int large = 0;
+#pragma unroll
+                for (int i = 0; i < NA; ++i) {
+                    int a[NC];
+                    upper(i, a);
+#pragma unroll
+                    for (int c = 0; c < NC; ++c) large += a[c] + (kLarge << 20) >= top[c] ? 1 << (16 * c) : 0;
+                }
+                large += __shfl_xor_sync(0xffffffffu, large, 1);
+                large += __shfl_xor_sync(0xffffffffu, large, 2);
+#pragma unroll
+                for (int c = 0; c < NC; ++c) slow = slow || (top[c] != 0 && ((large >> (16 * c)) & 0xffff) <= few);
+            }
 #pragma unroll
             for (int i = 0; i < NA; ++i) {
+                // off +- the magnitude, F half units of 2^-P, rounded to whole ones (truncated,
+                // the error doubles). With a bit to spare (HALF) the half units go along, and the
+                // shift in digits() drops them: downwards, so a positive number first gets another
                 auto fixed = [&](double w, int e) {
                     const int hi = __double2hiint(w);
-                    const uint64_t F = shr64(mant64(hi, __double2loint(w)), (uint32_t)(64 - P + e - ((hi >> 20) & 0x7ff)));
-                    return hi < 0 ? off - F : off + F;
+                    const uint64_t F = shr64(mant64(hi, __double2loint(w)), (uint32_t)(63 - P + e - ((hi >> 20) & 0x7ff)));
+                    if constexpr (HALF) return hi < 0 ? 2 * off - F : 2 * off + 1 + F;
+                    else return hi < 0 ? off - ((F + 1) >> 1) : off + ((F + 1) >> 1);
                 };
                 int er = E[0], ej = E[0];
                 if constexpr (SPLIT) by_class(pcol, 4 * i + q, E[0], E[NC - 1], er, ej);
                 const uint64_t fr = fixed(v[i].x, er), fj = fixed(v[i].y, ej);
 #pragma unroll
-                for (int d = 0; d < ND; ++d) b[i][d] = digits<ND, B>(fr, fj, d);
+                for (int d = 0; d < ND; ++d) b[i][d] = digits<ND, B, HALF>(fr, fj, d);
             }
         }
         bool store = valid && !slow && !zero;
@@ -726,6 +758,19 @@ MatRange range_of(const double *mat, int entries) {
     }
     r.dm = r.em - lo;
     return r;
+}
+
+// the most entries of a row that are below 2^(em - 1 - bits)
+int small_entries(const double *mat, int k, int em, int bits) {
+    const int D = 1 << k;
+    const double line = std::ldexp(1.0, em - 1 - bits);
+    int most = 0;
+    for (int j = 0; j < D; ++j) {
+        int n = 0;
+        for (int i = j * D; i < (j + 1) * D; ++i) n += std::fmax(std::fabs(mat[2 * i]), std::fabs(mat[2 * i + 1])) < line;
+        most = std::max(most, n);
+    }
+    return most;
 }
 
 // round(v 2^(bits - em)) for |v| < 2^em
@@ -848,13 +893,14 @@ cudaError_t run_fx3(const LaunchCtx &L, void *sv, uint64_t n_groups, const Group
 
 template <int K>
 cudaError_t run_fxt(const LaunchCtx &L, void *sv, uint64_t n_groups, const GroupGeom &G, const int *tpos,
-                    const double *mat, const MatRange &r, void *d_mat) {
+                    const double *mat, const MatRange &r, int few, void *d_mat) {
     using Cfg = FxtCfg<K>;
     Offs<K> O;
     offsets<K>(tpos, O);
     const Parts parts = parts_of(mat, K);
     auto fill = [&](auto &M) {
         M.em = r.em;
+        M.few = few;
         M.parts = parts;
         for (int i = 0; i < (1 << (2 * K)); ++i) {
             for (int c = 0; c < 2; ++c) M.m[i][c] = (long long)to_fixed(mat[2 * i + c], r.em, Cfg::P);
@@ -894,20 +940,24 @@ bool try_dense_fx(const LaunchCtx &L, void *sv, int n, const GroupGeom &G, const
     if (k > 5) return false;
     const MatRange r = range_of(mat, 1 << (2 * k));
     if (!r.finite || r.em < -100 || r.em > 100) return false;
-    // The lines are where each layout's error bound ends (above), not where the times
-    // cross: the first that may run is the fastest. 26 qubits, ms: two limbs 0.32 / 0.44
-    // (k = 1, 2), digits 0.75 / 0.90 / 2.0 (k = 3, 4, 5), three limbs 1.02 / 2.98 (k = 2,
-    // 4), FP64 1.02 / 2.03 / 4.06 / 8.1 / 14.0. k = 6 stays in FP64.
+    // The lines are where each layout's error reaches FP64's (above), not where the times
+    // cross: the first that may run is the fastest. 26 qubits, ms: two limbs 0.32 / 0.45
+    // (k = 1, 2), digits 0.79 / 0.91 / 2.0 (k = 3, 4, 5), three limbs 0.79 / 0.99 / 1.59 /
+    // 2.98 (k = 1 to 4), FP64 1.03 / 2.05 / 4.08 / 8.1 / 14.0. k = 6 stays in FP64.
     const uint64_t n_groups = 1ull << (n - G.ns);
-    if (k <= 2 && !r.zeros && r.dm <= (k == 1 ? 6 : 5)) {
+    if (k <= 2 && !r.zeros && r.dm <= (k == 1 ? 5 : 4)) {
         e = k == 1 ? run_fx2<1>(L, sv, n_groups, G, tpos, mat, r.em) : run_fx2<2>(L, sv, n_groups, G, tpos, mat, r.em);
         return true;
     }
     if (k >= 3 && !r.zeros && r.dm <= (k == 5 ? 11 : 8)) {
-        e = k == 3   ? run_fxt<3>(L, sv, n_groups, G, tpos, mat, r, d_mat)
-            : k == 4 ? run_fxt<4>(L, sv, n_groups, G, tpos, mat, r, d_mat)
-                     : run_fxt<5>(L, sv, n_groups, G, tpos, mat, r, d_mat);
-        return true;
+        const int sure = k == 5 ? 8 : 7;
+        const int few = r.dm <= sure ? 0 : small_entries(mat, k, r.em, sure - kLarge);
+        if (few <= (1 << k) / 2) {
+            e = k == 3   ? run_fxt<3>(L, sv, n_groups, G, tpos, mat, r, few, d_mat)
+                : k == 4 ? run_fxt<4>(L, sv, n_groups, G, tpos, mat, r, few, d_mat)
+                         : run_fxt<5>(L, sv, n_groups, G, tpos, mat, r, few, d_mat);
+            return true;
+        }
     }
     if (k > 4 || r.dm > 16) return false;
     switch (k) {

@@ -1,5 +1,9 @@
-"""complex128 dense gates in block fixed point (csrc/k_dense_fx.cu) where its groups are uneven (u = 2^-53).
+"""complex128 dense gates in block fixed point (csrc/k_dense_fx.cu) where their ranges end.
 
+Spread: matrices whose small entries meet the large amplitudes of a group are held, amplitude by amplitude, to 1.25
+times the worst error of the FP64 chain that the kernel stands in for, on the same groups (both as multiples of
+u sum |m||x|, u = 2^-53; the quarter is for the maximum of a few thousand groups being itself a random number), and
+never below 3 u for the closing roundings.
 Parts: a matrix whose entries are all real, or that becomes so when some rows and columns are multiplied by i, adds
 nothing from one half of a group's parts to the other. Each part is held to 2 (2 * 2^k + 2) u of its own sum."""
 import numpy as np
@@ -12,6 +16,18 @@ pytestmark = pytest.mark.gpu
 LD = np.longdouble
 
 
+def chain(m, x):
+    """One chain of FP64 multiply-adds per part, members in order."""
+    def fma(a, b, c):
+        return (a.astype(LD) * b.astype(LD) + c.astype(LD)).astype(np.float64)
+
+    re = im = np.zeros(x.shape)
+    for a, b in zip(m.T[:, :, None], x[:, None, :]):
+        re = fma(-a.imag, b.imag, fma(a.real, b.real, re))
+        im = fma(a.imag, b.real, fma(a.real, b.imag, im))
+    return re, im
+
+
 def exact(m, x):
     mr, mi, a, b = (p.astype(LD) for p in (m.real, m.imag, x.real, x.imag))
     return mr @ a - mi @ b, mr @ b + mi @ a
@@ -22,6 +38,36 @@ def run(m, x):
     k = m.shape[0].bit_length() - 1
     out = apply(np.ascontiguousarray(x.T).reshape(-1), tuple(range(k)), m).reshape(-1, 1 << k).T
     return out.real, out.imag
+
+
+def worst(got, want, scale):
+    err = np.hypot(*(np.abs(g - w).astype(float) for g, w in zip(got, want)))
+    return np.max(err / scale) / U
+
+
+def spread_matrix(rng, k, dm, small):
+    """Entries near the largest, but the first `small` columns' exponents dm below it."""
+    d = 1 << k
+    m = rng.uniform(.5, 1, (d, d)) * rng.choice([-1, 1], (d, d)) + 1j * rng.uniform(.5, 1, (d, d)) * rng.choice([-1, 1], (d, d))
+    m[:, :small] = (0.5 + 0.02 * rng.random((d, small))) * 2.0 ** -dm * (1 + 1j * rng.uniform(-1, 1, (d, small)))
+    return m
+
+
+@pytest.mark.parametrize("k", [1, 2, 3, 4, 5])
+@pytest.mark.parametrize("dm", [4, 5, 6, 7, 8, 11, 12, 17])
+@pytest.mark.parametrize("depth", [3, 9, 14, 30])
+def test_small_entries_meet_large_amplitudes(k, dm, depth):
+    rng = gen.rng_for(100 * k + dm)
+    d, count = 1 << k, 4096 >> max(0, k - 3)
+    for small in sorted({1, d // 2}):
+        m = spread_matrix(rng, k, dm, small)
+        for large in sorted({1, small, min(small + 1, d)}):
+            x = (rng.standard_normal((d, count)) + 1j * rng.standard_normal((d, count))) * 2.0 ** -depth
+            x[:large] = rng.uniform(.5, 1, (large, count)) + 1j * rng.uniform(-1, 1, (large, count))
+            want, scale = exact(m, x), np.abs(m) @ np.abs(x)
+            here, fp64 = worst(run(m, x), want, scale), worst(chain(m, x), want, scale)
+            print(f"small {small}, large {large}: {here:.2f} u, FP64 {fp64:.2f} u")
+            assert here <= 1.25 * max(fp64, 2.4), (small, large, here, fp64)
 
 
 def real_like(rng, k):
