@@ -64,7 +64,9 @@ inline cudaError_t launch_dependent(void (*kern)(P...), unsigned grid, unsigned 
     attr.val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kern, std::forward<A>(args)...);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, std::forward<A>(args)...);
+    if (e != cudaSuccess) cudaGetLastError();   // reported here, not by the next launch that asks
+    return e;
 }
 
 template <int K> struct Offs { uint64_t o[1 << K]; };
