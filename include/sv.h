@@ -67,7 +67,15 @@ typedef enum {
 } sv_status_t;
 
 /* Arithmetic of fused gates of 5-6 qubits on a complex64 state (Sec. II-B).
- * NATIVE: FP32 complex arithmetic on CUDA cores.
+ * NATIVE: the state's own precision, as for every other gate. complex64: FP32
+ *   complex arithmetic on CUDA cores, or for 5-6 qubits on 22 and more (without
+ *   controls, entries of a row within 2^11 of each other) BF16 digits on the
+ *   tensor cores whose error is no larger; there a non-finite amplitude makes its
+ *   group NaN. complex128: FP64 complex arithmetic, or fixed point with an error
+ *   of each amplitude's modulus no larger than FP64's, in u sum |m||x| over the
+ *   amplitudes it is formed from. A real or imaginary part far below its
+ *   amplitude carries the error of the modulus, except under matrices that keep
+ *   the parts apart (real, or real up to factors i of rows and columns).
  * TF32: tensor cores, operands rounded to TF32, FP32 accumulation.
  * SPLIT_BF16: tensor cores, each operand split into a BF16 high and low part,
  *   three products (hi*hi + hi*lo + lo*hi), FP32 accumulation. */
@@ -211,11 +219,13 @@ SV_API sv_status_t sv_fuse_plan_ex(const sv_gate_t *gates, int n_gates, int n_qu
  * out[s] = Re <psi| P_s |psi>, P_s = prod_i paulis[s*n_sites + i] on qubit
  * sites[s*n_sites + i]. Not divided by <psi|psi>. Products are formed in the
  * state's precision. complex128: accumulated in FP64. complex64: each thread
- * adds up to 8 terms in FP32, accumulates those partials in FP32 with
- * compensation (Neumaier), and everything across threads and blocks is
- * summed in FP64 in a fixed order (bitwise reproducible); the absolute error
- * stays below about 1.2e-6 <psi|psi> (the terms' magnitudes sum to at most
- * <psi|psi>) and is typically far smaller. out is host memory of n_strings
+ * adds up to 16 pairs (or 32 squares) in FP32 as a tree, accumulates those
+ * partials in FP32 with compensation (Neumaier), and everything across threads
+ * and blocks is summed in FP64; the absolute error stays below about 1.2e-6
+ * <psi|psi> (the terms' magnitudes sum to at most <psi|psi>) and is typically far
+ * smaller. Strings share passes, and the order of a string's sum follows from all
+ * strings of the call: the same list gives the same bits, a string in another
+ * list the same value within that error. out is host memory of n_strings
  * doubles. Synchronises the stream. Errors: INVALID_ARGUMENT for a site outside
  * [0, n), a site repeated within a string, a code outside 0..3. */
 SV_API sv_status_t sv_expectation_pauli(sv_handle_t h, const int *paulis, const int *sites,
@@ -259,7 +269,8 @@ SV_API sv_status_t sv_apply_pauli_rotation(sv_handle_t h, double theta, const in
 /* Sampler (Table I, "Sampler"): measurement outcomes of all qubits without
  * collapsing the state. For each randnums[t] in [0, 1), out[t] is the basis
  * index i at which the cumulative probability sum_{k<=i} |psi_k|^2 first
- * exceeds randnums[t] * <psi|psi> (probabilities summed in FP64). out is host
+ * exceeds randnums[t] * <psi|psi> (complex64: FP32 sums of 16 probabilities, FP64
+ * beyond). out is host
  * memory of n_samples int64. Synchronises the stream. Errors:
  * INVALID_ARGUMENT for a random number outside [0, 1) or NULL pointers. */
 SV_API sv_status_t sv_sample(sv_handle_t h, const double *randnums, int n_samples, int64_t *out);
@@ -284,7 +295,10 @@ SV_API sv_status_t sv_measure(sv_handle_t h, const int *qubits, int n_qubits, do
 SV_API sv_status_t sv_norm2(sv_handle_t h, double *out);
 
 /* Synchronise the stream and report whether a bounded device-side wait gave
- * up since the last call (SV_ERR_TIMEOUT), then clear the flag. */
+ * up since the last call (SV_ERR_TIMEOUT), then clear the flag. The gates on 5-6
+ * qubits of a complex64 state that run on the tensor cores have such waits, also
+ * in NATIVE precision; after a timeout (about 2 s: the GPU is not working as it
+ * should) the state is not valid, and this call alone says so. */
 SV_API sv_status_t sv_check_device_status(sv_handle_t h);
 
 /* Diagnostic of device-side failure detection: launch one wait that nothing

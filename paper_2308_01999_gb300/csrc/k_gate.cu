@@ -10,9 +10,9 @@
 //                registers, the matrix broadcast from shared memory;
 //   k_dense6     the same for k = 6, a group over a pair of lanes;
 //   k_dense_smem dense product for any k <= 6, a tile of groups staged in shared memory
-//                (complex128, and states of fewer than 16 groups; for k = 5, 6 the work
-//                is ALU-bound on CUDA cores; the tensor-core path in k_tc.cu is the
-//                fast one);
+//                (complex128 with k = 5, 6 and states of fewer than 16 groups);
+// (The dispatch here is what is left by k_tc_x3.cu -- complex64, k = 5, 6 on large
+// states -- and k_dense_fx.cu -- complex128, k <= 5, fixed point instead of FP64.)
 //   k_diag       diagonal matrix on the amplitudes where the controls hold;
 //   k_perm       generalized permutation matrix (one nonzero per row/column).
 //
