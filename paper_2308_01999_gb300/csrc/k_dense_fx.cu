@@ -465,14 +465,14 @@ k_dense_fx3(double2 *__restrict__ sv, uint64_t n_groups, GroupGeom G, const __gr
 }
 
 // ---------------------------------------------------------------------------
-// k = 3, 4, 5 on the tensor cores, for matrices with no zero entry. Fixed point of P bits, rounded (truncated, the worst
-// amplitude had twice the error), in ND balanced digits of B bits, held as FP16
-// integers; a group's 2 2^k reals are one column of an mma.sync B operand, the
+// k = 3, 4, 5 on the tensor cores, for matrices with no zero entry. Fixed point of P
+// bits, rounded (truncated, the worst amplitude had twice the error), in ND balanced
+// digits of B bits, held as FP16 integers; a group's 2 2^k reals are one column of an mma.sync B operand, the
 // matrix (real 2 x 2 blocks) is A, and digit products of equal weight are summed
 // by the FP32 accumulators, exactly: |digit| <= 2^(B-1), so a sum of 2 2^k terms
 // and up to ND digit pairs stays within 2^24, where every integer is an FP32 number
-// (that the accumulation then rounds nothing is not documented; full sums of largest
-// digits are among the tests):
+// (that the accumulation then rounds nothing is not documented: it rests on the tests,
+// which have sums of largest digits, and such sums that cancel):
 //   k = 3, 4: 7 digits of 9 bits, 2^16 * 32 * 7 = 2^23.8
 //   k = 5:    8 digits of 8 bits, 2^14 * 64 * 8 = 2^23
 // Products of digits i, j (from the top) with i + j > ND are left out: below
@@ -888,7 +888,8 @@ cudaError_t run_fx3(const LaunchCtx &L, void *sv, uint64_t n_groups, const Group
     constexpr int S = K >= 4 ? 2 : 1;
     ++*L.launches;
     return launch_dependent(M.parts.split ? k_dense_fx3<K, S, true> : k_dense_fx3<K, S, false>,
-                            (unsigned)((n_groups * S + kFx3Threads - 1) / kFx3Threads), kFx3Threads, 0, L.stream, reinterpret_cast<double2 *>(sv), n_groups, G, O, M);
+                            (unsigned)((n_groups * S + kFx3Threads - 1) / kFx3Threads), kFx3Threads, 0, L.stream,
+                            reinterpret_cast<double2 *>(sv), n_groups, G, O, M);
 }
 
 template <int K>

@@ -33,17 +33,18 @@
 // from and store it. Tiles are 64 columns (32 KiB), in four stages. The matrix is in
 // TMEM, beside the accumulators, because the shared-memory port is what the roles
 // share. The twelve small kinds of two tiles have an accumulator each, so the next
-// tile's can run while the epilogue reads this one (with one: 1.46 ms a gate, 1.13 so).
+// tile's can run while the epilogue reads this one (with one: 1.46 ms a gate, 1.11 so).
 //
 // A 5-target gate takes one more qubit as the top member bit with an identity:
 // the block-diagonal product keeps its halves apart, and each half of a column
 // has its own X.
 //
-// What bounds it: the tensor pipe, busy 3430 clocks per tile of 64 columns (52 MMAs),
-// and the conversion that feeds it, of about 5200 in all; HBM needs 3000. 28 qubits,
-// one gate: 1.13 to 1.16 ms for k = 6 (k_dense6 3.30) and 1.08 to 1.10 ms for k = 5
-// (k_dense5 1.40); 1.17 to 1.21 and 1.13 to 1.15 ms with qubit 0 a target (3.24 and
-// 1.36). N = 64 MMAs (half-tile accumulators) take as long as N = 128 ones; digits by
+// What bounds it: the tensor pipe, active 3430 of the 4800 clocks of a tile of 64
+// columns (52 MMAs; the thread that issues them waits for operands or accumulators in
+// 4 % of the time, and shared memory serves their operands beside the other roles);
+// HBM needs 3000. 28 qubits, one gate: 1.10 to 1.12 ms for k = 6 (k_dense6 3.30) and
+// 1.05 to 1.10 ms for k = 5 (k_dense5 1.38); 1.16 and 1.10 ms with qubit 0 a target
+// (3.24 and 1.34). N = 64 MMAs (half-tile accumulators) take as long as N = 128 ones; digits by
 // 4 convert warps instead of 8 that hold their atoms in registers, the matrix in shared
 // memory and ragged tiles were each slower.
 #include <cuda_bf16.h>

@@ -4,6 +4,9 @@ Spread: matrices whose small entries meet the large amplitudes of a group are he
 times the worst error of the FP64 chain that the kernel stands in for, on the same groups (both as multiples of
 u sum |m||x|, u = 2^-53; the quarter is for the maximum of a few thousand groups being itself a random number), and
 never below 3 u for the closing roundings.
+Full sums: largest digits of one sign, whose sums come near 2^24 units, stay within 2 u, and cancel where half of them
+change sign, to what the kernel states that it leaves out (2^-65 of the sum of magnitudes; a sum of digits that is off
+by one unit would show as 2^-50).
 Parts: a matrix whose entries are all real, or that becomes so when some rows and columns are multiplied by i, adds
 nothing from one half of a group's parts to the other. Each part is held to 2 (2 * 2^k + 2) u of its own sum."""
 import numpy as np
@@ -68,6 +71,24 @@ def test_small_entries_meet_large_amplitudes(k, dm, depth):
             here, fp64 = worst(run(m, x), want, scale), worst(chain(m, x), want, scale)
             print(f"small {small}, large {large}: {here:.2f} u, FP64 {fp64:.2f} u")
             assert here <= 1.25 * max(fp64, 2.4), (small, large, here, fp64)
+
+
+@pytest.mark.parametrize("k", [3, 4, 5])
+@pytest.mark.parametrize("digit", [8, 9])
+def test_full_sums_of_digits(k, digit):
+    d = 1 << k
+    bits = "1" * (digit - 2)                                            # the top digit, then digits of all ones below their sign
+    while len(bits) < 53:
+        bits += "0" + "1" * (digit - 1)
+    a = int(bits[:53], 2) * 2.0 ** -53
+    m = np.full((d, d), a - 1j * a)
+    m[1::2] = a + 1j * a                                                # these rows' imaginary parts add up, the others' real parts
+    x = np.full((d, 8), a + 1j * a)
+    x[d // 2:, 1::2] *= -1
+    want, got = exact(m, x), run(m, x)
+    left_out = 2.0 ** -65 * (np.abs(m) @ np.abs(x))
+    for w, g in zip(want, got):
+        assert np.all(np.abs(g - w).astype(float) <= 2 * U * np.abs(w).astype(float) + left_out)
 
 
 def real_like(rng, k):
