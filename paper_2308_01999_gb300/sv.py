@@ -402,19 +402,21 @@ class StateVector:
         sv_apply_matrix(self.handle, g.targets, g.matrix, g.controls, g.control_values or None, adjoint)
 
     def apply_circuit(self, gates):
-        """A list or tuple of gates in one native call; other iterables gate by gate, each asked for its next
-        gate after the one before has been applied (a generator may look at the state)."""
-        arr = None
-        if isinstance(gates, (list, tuple)) and type(self).apply_gate is StateVector.apply_gate:
-            try:
-                arr, _keep = _gate_array(gates, square=True)
-            except Exception:       # a gate that cannot be packed: the ones before it still apply
-                pass
-        if arr is None:
+        """A list or tuple of gates in native calls of many gates each; other iterables gate by gate, each asked
+        for its next gate after the one before has been applied (a generator may look at the state)."""
+        if not isinstance(gates, (list, tuple)) or type(self).apply_gate is not StateVector.apply_gate:
             for g in gates:
                 self.apply_gate(g)
             return
-        _check(lib().sv_apply_circuit(_VP(self.handle), arr, len(gates)), "sv_apply_circuit")
+        for begin in range(0, len(gates), 512):         # the packed copies stay small: at most 32 MiB of matrices
+            part = gates[begin:begin + 512]
+            try:
+                arr, _keep = _gate_array(part, square=True)
+            except Exception:       # a gate that cannot be packed: the ones before it still apply
+                for g in part:
+                    self.apply_gate(g)
+                continue
+            _check(lib().sv_apply_circuit(_VP(self.handle), arr, len(part)), "sv_apply_circuit")
 
     def apply_fused(self, gates, max_fused_qubits: int, prec: int = SV_PREC_NATIVE,
                     max_fused_diagonal_qubits: int = 0) -> int:

@@ -56,3 +56,37 @@ def test_overridden_apply_gate_is_called(state):
     state.__class__ = Counting
     state.apply_circuit([gen.Gate((0,), X), gen.Gate((1,), np.eye(2))])
     assert state.log == [(0,), (1,)]
+
+
+def test_long_lists_are_packed_in_parts(state, monkeypatch):
+    """The packed copies of the matrices stay bounded, whatever the circuit's length; the order is kept."""
+    calls = []
+
+    class Lib:
+        @staticmethod
+        def sv_apply_circuit(h, gates, n):
+            calls.append([gates[i].targets[0] for i in range(n)])
+            return 0
+
+    monkeypatch.setattr(sv, "lib", lambda: Lib)
+    order = [i % 7 for i in range(10001)]
+    state.apply_circuit([gen.Gate((q,), X) for q in order])
+    assert sum(calls, []) == order
+    assert max(map(len, calls)) <= 4096
+    wide = gen.Gate(tuple(range(6)), np.eye(64))
+    calls.clear()
+    state.apply_circuit((wide,) * 600)
+    assert sum(map(len, calls)) == 600 and max(map(len, calls)) * 64 * 64 * 16 <= 1 << 25
+
+
+def test_gate_that_cannot_be_packed_in_a_later_part(state, monkeypatch):
+    class Lib:
+        @staticmethod
+        def sv_apply_circuit(h, gates, n):
+            state.log.extend(("apply", (gates[i].targets[0],)) for i in range(n))
+            return 0
+
+    monkeypatch.setattr(sv, "lib", lambda: Lib)
+    gates = [gen.Gate((i % 5,), X) for i in range(5000)]
+    state.apply_circuit(gates + [gen.Gate((0,) * 24, X), gen.Gate((3,), X)])   # the recorder takes everything
+    assert [t for _, t in state.log[:5000]] == [g.targets for g in gates] and len(state.log) == 5002
