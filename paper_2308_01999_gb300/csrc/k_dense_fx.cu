@@ -23,9 +23,9 @@
 // than a chain of FP64 multiply-adds on the same groups; worst measured here / chain:
 //   k = 1, dm 5: 2.5 / 3.0   k = 2, dm 4: 3.7 / 4.8   (k = 2 at 5: 9.5 / 4.8)
 //   k = 3, dm 7: 5.3 / 7.1   k = 4, dm 7: 8.9 / 9.9   k = 5, dm 8: 12.0 / 14.2
-// Beyond that, up to 8 (k = 5: 11), the digits serve groups in which more amplitudes
-// are large than any row has small entries; then every sum sees a large one through a
-// large entry. Three limbs: host and kernel check that entries (dm bits) and nonzero
+// Beyond that, up to 8 (k = 5: 11), the digits serve groups in which every row sees a
+// large amplitude through a large entry, and (8; k = 5: 9) those whose reals, and then
+// all products, they hold exactly. Three limbs: host and kernel check that entries (dm bits) and nonzero
 // amplitudes (t bits) lie within t + dm <= 24 bits of their largest, which keeps the
 // error of every term below u / 16 of it. Zeros are exact throughout.
 //
@@ -507,7 +507,10 @@ template <int K> struct Fxt {
     long long m[1 << (2 * K)][2];   // round(2^(P - em) re, im)
     double2 f[1 << (2 * K)];        // for groups out of range
     int em;
-    int few;                        // a row's small entries, at most: as many large amplitudes do not bound every sum
+    int exact;                      // 0: every group may be computed so. Else groups whose reals lie within 2^exact
+                                    // are held exactly (negative: none), and the others need every row to see
+                                    // a large amplitude through an entry outside its
+    uint32_t small[1 << K];         // the small entries of each row
     Parts parts;
 };
 
@@ -551,7 +554,8 @@ k_dense_fxt(double2 *__restrict__ sv, uint64_t n_groups, GroupGeom G, const __gr
     const double2 *Mf = K <= 4 ? reinterpret_cast<const double2 *>(Mp.f) : Mg->f;
     let_next_start();
     if constexpr (K > 4) wait_for_previous();          // the matrix is in the workspace
-    const int em = K <= 4 ? Mp.em : Mg->em, few = K <= 4 ? Mp.few : Mg->few;
+    const int em = K <= 4 ? Mp.em : Mg->em, exact = K <= 4 ? Mp.exact : Mg->exact;
+    const uint32_t *small = K <= 4 ? Mp.small : Mg->small;
     const uint32_t prow = K <= 4 ? Mp.parts.row : Mg->parts.row, pcol = K <= 4 ? Mp.parts.col : Mg->parts.col;
     // A's fragments: lane 4 r + q holds rows r (re of member r) and r + 8 (its im),
     // members q (registers x, y) and q + 4 (z, w) of the step
@@ -622,20 +626,49 @@ k_dense_fxt(double2 *__restrict__ sv, uint64_t n_groups, GroupGeom G, const __gr
                 slow = slow || ((SPLIT ? top[c] != 0 : !zero) && out_of_range(top[c] >> 20));
                 E[c] = top[c] != 0 ? top[c] >> 20 : kEMin;   // zeros take any scale
             }
-            if (few) {
-                // large amplitudes (or reals of a class), in a half-word each
-                int large = 0;
+            if (exact) {
+                // a row all of whose large amplitudes (or reals of a class) meet small entries, in a
+                // group that is not held exactly
+                uint32_t large[NC], low[NC], lost = 0;
+#pragma unroll
+                for (int c = 0; c < NC; ++c) {
+                    large[c] = 0;
+                    low[c] = 0xffffffffu;
+                }
 #pragma unroll
                 for (int i = 0; i < NA; ++i) {
                     int a[NC];
                     upper(i, a);
+                    const uint32_t r = (uint32_t)(__double2hiint(v[i].x) & 0x7fffffff) - 1u;   // zeros wrap around
+                    const uint32_t j = (uint32_t)(__double2hiint(v[i].y) & 0x7fffffff) - 1u;
+                    uint32_t l[NC];
+                    if constexpr (SPLIT) by_class(pcol, 4 * i + q, r, j, l[0], l[NC - 1]);
+                    else l[0] = min(r, j);
 #pragma unroll
-                    for (int c = 0; c < NC; ++c) large += a[c] + (kLarge << 20) >= top[c] ? 1 << (16 * c) : 0;
+                    for (int c = 0; c < NC; ++c) {
+                        low[c] = min(low[c], l[c]);
+                        if (a[c] + (kLarge << 20) >= top[c]) large[c] |= 1u << (4 * i + q);
+                    }
                 }
-                large += __shfl_xor_sync(0xffffffffu, large, 1);
-                large += __shfl_xor_sync(0xffffffffu, large, 2);
 #pragma unroll
-                for (int c = 0; c < NC; ++c) slow = slow || (top[c] != 0 && ((large >> (16 * c)) & 0xffff) <= few);
+                for (int o = 1; o < 4; o <<= 1) {
+#pragma unroll
+                    for (int c = 0; c < NC; ++c) {
+                        low[c] = min(low[c], __shfl_xor_sync(0xffffffffu, low[c], o));
+                        large[c] |= __shfl_xor_sync(0xffffffffu, large[c], o);
+                    }
+                }
+                for (int row = q; row < D; row += 4) {
+                    const uint32_t s = small[row];
+#pragma unroll
+                    for (int c = 0; c < NC; ++c) lost |= (large[c] & ~s) == 0 ? 1u << c : 0u;
+                }
+                lost |= __shfl_xor_sync(0xffffffffu, lost, 1);
+                lost |= __shfl_xor_sync(0xffffffffu, lost, 2);
+#pragma unroll
+                for (int c = 0; c < NC; ++c)
+                    slow = slow || (top[c] != 0 && ((lost >> c) & 1u) &&
+                                    (exact < 0 || (uint32_t)top[c] - low[c] > (uint32_t)exact << 20));
             }
 #pragma unroll
             for (int i = 0; i < NA; ++i) {
@@ -760,15 +793,18 @@ MatRange range_of(const double *mat, int entries) {
     return r;
 }
 
-// the most entries of a row that are below 2^(em - 1 - bits)
-int small_entries(const double *mat, int k, int em, int bits) {
+// row by row, the entries below 2^(em - 1 - bits); returns how many a row has at most
+int small_entries(const double *mat, int k, int em, int bits, uint32_t *rows) {
     const int D = 1 << k;
     const double line = std::ldexp(1.0, em - 1 - bits);
     int most = 0;
     for (int j = 0; j < D; ++j) {
-        int n = 0;
-        for (int i = j * D; i < (j + 1) * D; ++i) n += std::fmax(std::fabs(mat[2 * i]), std::fabs(mat[2 * i + 1])) < line;
-        most = std::max(most, n);
+        rows[j] = 0;
+        for (int l = 0; l < D; ++l) {
+            const double *m = mat + 2 * (j * D + l);
+            if (std::fmax(std::fabs(m[0]), std::fabs(m[1])) < line) rows[j] |= 1u << l;
+        }
+        most = std::max(most, __builtin_popcount(rows[j]));
     }
     return most;
 }
@@ -894,14 +930,15 @@ cudaError_t run_fx3(const LaunchCtx &L, void *sv, uint64_t n_groups, const Group
 
 template <int K>
 cudaError_t run_fxt(const LaunchCtx &L, void *sv, uint64_t n_groups, const GroupGeom &G, const int *tpos,
-                    const double *mat, const MatRange &r, int few, void *d_mat) {
+                    const double *mat, const MatRange &r, int exact, const uint32_t *small, void *d_mat) {
     using Cfg = FxtCfg<K>;
     Offs<K> O;
     offsets<K>(tpos, O);
     const Parts parts = parts_of(mat, K);
     auto fill = [&](auto &M) {
         M.em = r.em;
-        M.few = few;
+        M.exact = exact;
+        std::copy(small, small + Cfg::D, M.small);
         M.parts = parts;
         for (int i = 0; i < (1 << (2 * K)); ++i) {
             for (int c = 0; c < 2; ++c) M.m[i][c] = (long long)to_fixed(mat[2 * i + c], r.em, Cfg::P);
@@ -951,12 +988,18 @@ bool try_dense_fx(const LaunchCtx &L, void *sv, int n, const GroupGeom &G, const
         return true;
     }
     if (k >= 3 && !r.zeros && r.dm <= (k == 5 ? 11 : 8)) {
-        const int sure = k == 5 ? 8 : 7;
-        const int few = r.dm <= sure ? 0 : small_entries(mat, k, r.em, sure - kLarge);
-        if (few <= (1 << k) / 2) {
-            e = k == 3   ? run_fxt<3>(L, sv, n_groups, G, tpos, mat, r, few, d_mat)
-                : k == 4 ? run_fxt<4>(L, sv, n_groups, G, tpos, mat, r, few, d_mat)
-                         : run_fxt<5>(L, sv, n_groups, G, tpos, mat, r, few, d_mat);
+        const int sure = k == 5 ? 8 : 7, spare = k == 5 ? 9 : 8;     // spare: bits beyond a double's 53
+        uint32_t small[32] = {0};
+        int exact = 0;
+        bool ok = true;
+        if (r.dm > sure) {
+            exact = r.dm <= spare ? spare : -1;
+            ok = small_entries(mat, k, r.em, sure - kLarge, small) <= 3 * (1 << k) / 4;
+        }
+        if (ok) {
+            e = k == 3   ? run_fxt<3>(L, sv, n_groups, G, tpos, mat, r, exact, small, d_mat)
+                : k == 4 ? run_fxt<4>(L, sv, n_groups, G, tpos, mat, r, exact, small, d_mat)
+                         : run_fxt<5>(L, sv, n_groups, G, tpos, mat, r, exact, small, d_mat);
             return true;
         }
     }

@@ -58,7 +58,7 @@ def spread_matrix(rng, k, dm, small):
 
 @pytest.mark.parametrize("k", [1, 2, 3, 4, 5])
 @pytest.mark.parametrize("dm", [4, 5, 6, 7, 8, 11, 12, 17])
-@pytest.mark.parametrize("depth", [3, 9, 14, 30])
+@pytest.mark.parametrize("depth", [3, 9, 14, 30, 2000])
 def test_small_entries_meet_large_amplitudes(k, dm, depth):
     rng = gen.rng_for(100 * k + dm)
     d, count = 1 << k, 4096 >> max(0, k - 3)
@@ -71,6 +71,26 @@ def test_small_entries_meet_large_amplitudes(k, dm, depth):
             here, fp64 = worst(run(m, x), want, scale), worst(chain(m, x), want, scale)
             print(f"small {small}, large {large}: {here:.2f} u, FP64 {fp64:.2f} u")
             assert here <= 1.25 * max(fp64, 2.4), (small, large, here, fp64)
+
+
+@pytest.mark.parametrize("k", [1, 2, 3, 4, 5])
+@pytest.mark.parametrize("dm", [7, 8, 9, 10, 11])
+@pytest.mark.parametrize("real", [False, True])
+def test_small_entries_anywhere(k, dm, real):
+    """Small entries in any places, and groups with any of their amplitudes large, the others small or zero."""
+    rng = gen.rng_for(1000 * k + dm + real)
+    d, count = 1 << k, 4096 >> max(0, k - 3)
+    m = spread_matrix(rng, k, dm, 0)
+    m = np.where(rng.random((d, d)) < 0.3, 2.0 ** -dm * rng.uniform(0.9, 1, (d, d)), 1) * m
+    if real:
+        m = m.real + 0j
+    x = rng.uniform(.5, 1, (d, count)) + 1j * rng.uniform(-1, 1, (d, count))
+    x *= np.where(rng.random((d, count)) < rng.uniform(0, 1, count), 1, 2.0 ** -rng.choice([3, 14, 30, 2000], count).astype(float))
+    x[0, ~x.any(axis=0)] = 1
+    want, scale = exact(m, x), np.abs(m) @ np.abs(x)
+    here, fp64 = worst(run(m, x), want, scale), worst(chain(m, x), want, scale)
+    print(f"dm {dm}, real {real}: {here:.2f} u, FP64 {fp64:.2f} u")
+    assert here <= 1.25 * max(fp64, 2.4)
 
 
 @pytest.mark.parametrize("k", [3, 4, 5])
