@@ -18,8 +18,7 @@
 // of the whole product would shrink the norm by a constant per gate). The other
 // products (digits i, j from the top with i + j <= 4: 12 kinds) are at most 2^-7 of
 // the first, go into a second accumulator smallest first, and the two are added
-// with one rounding. Error per gate: see the
-// rule in tc_x3_ok(). Three state digits and nine products (0.98 to 1.00 ms a gate on
+// with one rounding. Error per gate: see the rule in tc_x3_ok(). Three state digits and nine products (0.98 to 1.00 ms a gate on
 // 28 qubits) kept 25 bits below X: where one amplitude dominates a group the small
 // outputs then had up to 700 u sum |m||x|.
 //
@@ -39,14 +38,14 @@
 // the block-diagonal product keeps its halves apart, and each half of a column
 // has its own X.
 //
-// What bounds it: the tensor pipe, active 3430 of the 4800 clocks of a tile of 64
-// columns (52 MMAs; the thread that issues them waits for operands or accumulators in
-// 4 % of the time, and shared memory serves their operands beside the other roles);
-// HBM needs 3000. 28 qubits, one gate: 1.10 to 1.12 ms for k = 6 (k_dense6 3.30) and
+// What bounds it: the conversion and the tensor pipe, each close to the 4800 clocks of
+// a tile of 64 columns (the convert warps wait in 15 % of them, the thread that issues
+// the 52 MMAs in 4 %, the pipe is active in 3430; with 10 or 11 products for matrices
+// that need no more, a gate was no faster); HBM needs 3000. 28 qubits, one gate: 1.10 to 1.12 ms for k = 6 (k_dense6 3.30) and
 // 1.05 to 1.10 ms for k = 5 (k_dense5 1.38); 1.16 and 1.10 ms with qubit 0 a target
-// (3.24 and 1.34). N = 64 MMAs (half-tile accumulators) take as long as N = 128 ones; digits by
-// 4 convert warps instead of 8 that hold their atoms in registers, the matrix in shared
-// memory and ragged tiles were each slower.
+// (3.24 and 1.34). N = 64 MMAs (half-tile accumulators) take as long as N = 128 ones;
+// digits by 4 convert warps instead of 8 that hold their atoms in registers, the matrix
+// in shared memory and ragged tiles were each slower.
 #include <cuda_bf16.h>
 
 #include <cmath>
