@@ -182,18 +182,23 @@ k_dense_fx2(double2 *__restrict__ sv, uint64_t n_groups, GroupGeom G, Offs<K> O,
                     any[0] |= ar | aj;
                 }
             }
-            if ((any[0] && out_of_range(E[0])) || (SPLIT && any[1] && out_of_range(E[1]))) {
+            const bool none = (any[0] | any[1]) == 0;      // most groups of a state near a basis state
+            if (none || (any[0] && out_of_range(E[0])) || (SPLIT && any[1] && out_of_range(E[1]))) {
 #pragma unroll
                 for (int j = 0; j < D; ++j) {
                     double2 acc = make_double2(0.0, 0.0);
+                    if (!none) {
 #pragma unroll
-                    for (int l = 0; l < D; ++l) cmad(acc, M.f[j * D + l], v[u][l]);
+                        for (int l = 0; l < D; ++l) cmad(acc, M.f[j * D + l], v[u][l]);
+                    }
                     sv[base[u] + O.o[j]] = acc;
                 }
                 continue;
             }
-            if (!any[0]) E[0] = kEMin;
-            if (!SPLIT || !any[1]) E[1] = kEMin;
+            if constexpr (SPLIT) {
+                if (!any[0]) E[0] = kEMin;
+                if (!any[1]) E[1] = kEMin;
+            }
         }
         int x1[2 * D], x0[2 * D];
 #pragma unroll
